@@ -18,7 +18,8 @@
 // Weights with rho |u_j| <= 8 u ||T|| (u = 2^-53, ||T|| the largest Gershgorin row sum) are
 // set to zero, the usual backward-stable deflation of divide and conquer; beyond the exact
 // deflation of Sec. 1 it keeps every surviving u_j^2 in the normal range of binary64.
-// The products run in k_dc_gemm, a binary64 tiled GEMM that reads W^T through pos.
+// The products run in k_dc_gemm, a binary64 tiled GEMM over the rows and positions that do not
+// deflate (DcAct); deflated rows are copied (k_dc_copy).
 // Storage per depth: eigenvalues in index order (n doubles), and each node's Q^T as an
 // N x N row-major block at voffs_t[i] = i q^2 + (2q + 1) floor(i r / 2^t), q = floor(n / 2^t),
 // r = n mod 2^t (the node sizes are q or q + 1, so the prefix sums of N^2 have this form).
@@ -225,19 +226,182 @@ __global__ void k_dc_merge(int64_t n, int t, const double* __restrict__ b, const
   }
 }
 
-// C = A B per node and half h (h = 0: columns 0..N1 with Q1; h = 1: columns N1..N with Q2):
-//   A[r, k] = W^T[r, pos(off_h + k)]  (N x N_h),  B = child's Q^T (N_h x N_h),
-//   C[r, c] -> Q^T_node[r, off_h + c].
-// One block computes a 64 x 64 tile of C with 256 threads (4 x 4 each), k in steps of 16.
+// The structure of a depth's W^T that the products use (arrays of the depth's batched workspace that
+// are free once its eigenpairs are written).  A position with a zero weight is deflated exactly
+// (Sec. 1): its row of W^T is the unit vector e_q and its column is zero in every other row.  So
+// such a row of Q^T is the child's row, a copy, and the products run over the other rows and the
+// positions with a non-zero weight only, in the same order (the terms left out are exact zeros, so
+// the sums' bits do not change).
+struct DcAct {
+  int* rowsrc;   // [n] per output row: the position q of a unit row, or -1
+  int* inv;      // [n] per merged position: its index in the children's concatenated order
+  int* rows;     // [n] per node: the rows that are not unit rows, increasing
+  int* ks;       // [n] per child: the indices (in the child) of the positions with a weight, increasing
+  int* kp;       // [n] and their merged positions
+  int* cnt;      // [3 P] per node: the lengths of rows and of the two children's ks
+  const unsigned* call;   // the call's status word
+};
+
+// Bits that leave a depth's eigenpairs (and the lists below) unwritten
+constexpr unsigned ST_FATAL_DC = ST_NONFINITE | ST_UNSORTED | ST_BADARG | ST_RHO;
+
+// rowsrc and inv (one thread per element; a problem with rho == 0 has W^T = I).  Each of a
+// problem's N rows belongs to one reduced or one deflated pair, so every rowsrc is written.
+__global__ void k_dc_rowsrc(int64_t n, int t, Ws w, const int* __restrict__ pos, DcAct a) {
+  if (*a.call & ST_FATAL_DC) return;
+  for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = d_node(g, n, t);
+    const int64_t lo = d_start(i, n, t);
+    const int k = (int)(g - lo);
+    a.inv[lo + pos[g]] = k;
+    if (w.pst[i] & PT_TRIVIAL) {
+      a.rowsrc[g] = k;
+      continue;
+    }
+    const int nr = w.nred[i], nd = w.ndefl[i];
+    if (k < nr) a.rowsrc[lo + (nd ? w.rpos[g] : k)] = -1;
+    if (k < nd) {
+      const int q = w.dlist[g];
+      a.rowsrc[lo + w.dpos[g]] = (w.src[lo + q] < 0) ? q : -1;
+    }
+  }
+}
+
+// One block per node: the lists of rows and of each child's indices, by prefix counts over chunks
+// of the block.
+__global__ void __launch_bounds__(1024) k_dc_lists(int64_t n, int t, Ws w, const int* __restrict__ pos, DcAct a) {
+  __shared__ int wsum[3][32];
+  const int64_t P = (int64_t)1 << t;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const bool fatal = (*a.call & ST_FATAL_DC) != 0;
+  for (int64_t i = blockIdx.x; i < P; i += gridDim.x) {
+    const int64_t lo = d_start(i, n, t), hi = d_start(i + 1, n, t), mid = d_start(2 * i + 1, n, t + 1);
+    const int N = fatal ? 0 : (int)(hi - lo), N1 = (int)(mid - lo);
+    const unsigned ps = w.pst[i];
+    const bool triv = (ps & PT_TRIVIAL) != 0, defl = (ps & PT_DEFLATE) != 0;
+    int c0 = 0, c1 = 0, c2 = 0;
+    for (int k0 = 0; k0 < N; k0 += blockDim.x) {
+      const int k = k0 + threadIdx.x;
+      int p = 0;
+      bool ar = false, ak = false;
+      if (k < N) {
+        ar = a.rowsrc[lo + k] < 0;
+        p = pos[lo + k];
+        ak = !triv && (!defl || w.src[lo + p] >= 0);
+      }
+      const bool a1 = ak && k < N1, a2 = ak && k >= N1;
+      const unsigned m0 = __ballot_sync(FULL, ar), m1 = __ballot_sync(FULL, a1), m2 = __ballot_sync(FULL, a2);
+      if (lane == 0) { wsum[0][wid] = __popc(m0); wsum[1][wid] = __popc(m1); wsum[2][wid] = __popc(m2); }
+      __syncthreads();
+      int b0 = c0, b1 = c1, b2 = c2;
+      for (int q = 0; q < nw; q++) {
+        if (q < wid) { b0 += wsum[0][q]; b1 += wsum[1][q]; b2 += wsum[2][q]; }
+        c0 += wsum[0][q]; c1 += wsum[1][q]; c2 += wsum[2][q];
+      }
+      const unsigned below = (1u << lane) - 1u;
+      if (ar) a.rows[lo + b0 + __popc(m0 & below)] = k;
+      if (a1) { const int e = b1 + __popc(m1 & below); a.ks[lo + e] = k; a.kp[lo + e] = p; }
+      if (a2) { const int e = b2 + __popc(m2 & below); a.ks[mid + e] = k - N1; a.kp[mid + e] = p; }
+      __syncthreads();
+    }
+    if (threadIdx.x == 0) { a.cnt[3 * i] = c0; a.cnt[3 * i + 1] = c1; a.cnt[3 * i + 2] = c2; }
+  }
+}
+
+// The unit rows of W^T: Q^T_node[r, :] is the child's row, zero in the other half (a warp per row).
+__global__ void __launch_bounds__(256) k_dc_copy(int64_t n, int t, const double* __restrict__ QTc,
+                                                 double* __restrict__ out, int64_t ldo_root, DcAct a) {
+  if (*a.call & ST_FATAL_DC) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t g = wid; g < n; g += nw) {
+    const int64_t i = d_node(g, n, t);
+    const int64_t lo = d_start(i, n, t), hi = d_start(i + 1, n, t);
+    const int N = (int)(hi - lo);
+    if (N < 2) continue;
+    const int q = a.rowsrc[g];
+    if (q < 0) continue;
+    const int N1 = (int)(d_start(2 * i + 1, n, t + 1) - lo), N2 = N - N1;
+    const int s = a.inv[lo + q];
+    if ((unsigned)s >= (unsigned)N) continue;
+    double* C = (t == 0) ? out + g * ldo_root : out + d_voff(i, n, t) + (g - lo) * N;
+    const double* src = (s < N1) ? QTc + d_voff(2 * i, n, t + 1) + (int64_t)s * N1
+                                 : QTc + d_voff(2 * i + 1, n, t + 1) + (int64_t)(s - N1) * N2;
+    const int c0 = (s < N1) ? 0 : N1, c1 = (s < N1) ? N1 : N;
+    for (int c = lane; c < N; c += 32) C[c] = (c >= c0 && c < c1) ? src[c - c0] : 0.0;
+  }
+}
+
+// Eigenvalues only: the merges above read the first and the last column of each node's Q^T and
+// nothing else, so only those two are formed.  A block of two warps takes 32 of a node's rows, one
+// warp per column; each lane sums its row over the list in k_dc_gemm's order (a sequential chain of
+// fma: the eigenvalues are the bits of a call with eigenvectors), from a 32 x 32 tile of W^T that the
+// warp loads along the rows.
+__global__ void __launch_bounds__(64) k_dc_edges(int64_t n, int t, int64_t tiles_per_node,
+                                                 const double* __restrict__ WT, const double* __restrict__ QTc,
+                                                 double* __restrict__ out, DcAct a) {
+  __shared__ double tile[2][32][33];
+  __shared__ double col[2][32];
+  if (*a.call & ST_FATAL_DC) return;
+  const int lane = threadIdx.x & 31, h = threadIdx.x >> 5;
+  const int64_t i = blockIdx.x / tiles_per_node;
+  const int r0 = (int)(blockIdx.x - i * tiles_per_node) * 32;
+  const int64_t lo = d_start(i, n, t), hi = d_start(i + 1, n, t), mid = d_start(2 * i + 1, n, t + 1);
+  const int N = (int)(hi - lo), N1 = (int)(mid - lo);
+  if (N < 2 || r0 >= N) return;
+  const int Nh = h ? N - N1 : N1, off = h ? N1 : 0;
+  // the child's first column (left child) or last column (right child), with its row stride Nh
+  const double* __restrict__ Q = QTc + d_voff(2 * i + h, n, t + 1) + (h ? Nh - 1 : 0);
+  const double* __restrict__ W = WT + d_voff(i, n, t);
+  double* __restrict__ C = out + d_voff(i, n, t) + (h ? N - 1 : 0);
+  // unit rows: the child's entry, or zero in the other half
+  if (r0 + lane < N) {
+    const int q = a.rowsrc[lo + r0 + lane];
+    if (q >= 0) {
+      const int s = a.inv[lo + q] - off;
+      C[(int64_t)(r0 + lane) * N] = ((unsigned)s < (unsigned)Nh) ? Q[(int64_t)s * Nh] : 0.0;
+    }
+  }
+  const int M = a.cnt[3 * i], K = a.cnt[3 * i + 1 + h];
+  if (r0 >= M) return;                                   // this warp's block has no listed rows
+  const int row = (r0 + lane < M) ? a.rows[lo + r0 + lane] : -1;
+  double acc = 0.0;
+  for (int k0 = 0; k0 < K; k0 += 32) {
+    const bool in = k0 + lane < K;
+    const int kp = in ? a.kp[lo + off + k0 + lane] : -1;
+    col[h][lane] = in ? Q[(int64_t)a.ks[lo + off + k0 + lane] * Nh] : 0.0;
+#pragma unroll 8
+    for (int r = 0; r < 32; r++) {
+      const int rr = __shfl_sync(FULL, row, r);
+      tile[h][r][lane] = (rr >= 0 && kp >= 0) ? W[(int64_t)rr * N + kp] : 0.0;
+    }
+    __syncwarp();
+    for (int k = 0; k < 32; k++) acc = __fma_rn(tile[h][lane][k], col[h][k], acc);
+    __syncwarp();
+  }
+  if (row >= 0) C[(int64_t)row * N] = acc;
+}
+
+// C = A B per node and half h (h = 0: columns 0..N1 with Q1; h = 1: columns N1..N with Q2), over the
+// node's list of rows and the child's list of indices:
+//   A[r, k] = W^T[rows[r], kp[k]],  B[k, c] = child's Q^T[ks[k], c],
+//   C[r, c] -> Q^T_node[rows[r], off_h + c].
+// One block computes a 64 x 64 tile of C with 256 threads (4 x 4 each), k in steps of 16.  The grid
+// covers the whole node (the lists' lengths are known on the device only); the blocks beyond the
+// rows end at once.  Bound by the binary64 pipe (99% busy on a full product), so the terms left out
+// are what there is to gain: a random T (a, b ~ U(-1, 1)) of order 4096, whose eigenvectors are
+// localised and whose merges deflate nearly everywhere, takes 7.98 ms against 81.3 with full
+// products; a T that deflates nowhere pays the lists and the copy kernel, some microseconds a depth.
 constexpr int GT = 64, GK = 16;
 
 __global__ void __launch_bounds__(256) k_dc_gemm(int64_t n, int t, int64_t tiles_per_node,
-                                                 const double* __restrict__ WT, const int* __restrict__ pos,
-                                                 const double* __restrict__ QTc, double* __restrict__ out,
-                                                 int64_t ldo_root) {
+                                                 const double* __restrict__ WT, const double* __restrict__ QTc,
+                                                 double* __restrict__ out, int64_t ldo_root, DcAct a) {
   __shared__ double As[GK][GT + 1];
   __shared__ double Bs[GK][GT];
-  __shared__ int ps[GK];
+  __shared__ int ps[GK], ss[GK], rs[GT];
+  if (*a.call & ST_FATAL_DC) return;
   const int64_t item = blockIdx.x;
   const int64_t i = item / tiles_per_node;
   int64_t loc = item - i * tiles_per_node;
@@ -246,7 +410,8 @@ __global__ void __launch_bounds__(256) k_dc_gemm(int64_t n, int t, int64_t tiles
   if (N < 2) return;
   const int64_t mid = d_start(2 * i + 1, n, t + 1);
   const int N1 = (int)(mid - lo), N2 = (int)(hi - mid);
-  const int tr_ = (N + GT - 1) / GT;
+  const int M = a.cnt[3 * i];
+  const int tr_ = (M + GT - 1) / GT;
   const int tc1 = (N1 + GT - 1) / GT, tc2 = (N2 + GT - 1) / GT;
   int h, Nh, off, tr, tc;
   if (loc < (int64_t)tr_ * tc1) { h = 0; Nh = N1; off = 0; tr = (int)(loc / tc1); tc = (int)(loc % tc1); }
@@ -255,9 +420,11 @@ __global__ void __launch_bounds__(256) k_dc_gemm(int64_t n, int t, int64_t tiles
     if (loc >= (int64_t)tr_ * tc2) return;
     h = 1; Nh = N2; off = N1; tr = (int)(loc / tc2); tc = (int)(loc % tc2);
   }
+  const int K = a.cnt[3 * i + 1 + h];
   const double* __restrict__ W = WT + d_voff(i, n, t);
   const double* __restrict__ Bm = QTc + d_voff(2 * i + h, n, t + 1);
-  const int* __restrict__ pl = pos + lo + off;
+  const int* __restrict__ kp = a.kp + lo + off;
+  const int* __restrict__ ks = a.ks + lo + off;
   double* C;
   int64_t ldc;
   if (t == 0) { C = out; ldc = ldo_root; }
@@ -265,23 +432,26 @@ __global__ void __launch_bounds__(256) k_dc_gemm(int64_t n, int t, int64_t tiles
   const int tid = threadIdx.x;
   const int ty = tid >> 4, tx = tid & 15;
   const int row0 = tr * GT, col0 = tc * GT;
+  if (tid < GT) rs[tid] = (row0 + tid < M) ? a.rows[lo + row0 + tid] : -1;
   double acc[4][4];
 #pragma unroll
   for (int p = 0; p < 4; p++)
 #pragma unroll
     for (int q = 0; q < 4; q++) acc[p][q] = 0.0;
-  for (int k0 = 0; k0 < Nh; k0 += GK) {
-    if (tid < GK) ps[tid] = (k0 + tid < Nh) ? pl[k0 + tid] : 0;
+  for (int k0 = 0; k0 < K; k0 += GK) {
+    if (tid < GK) {
+      ps[tid] = (k0 + tid < K) ? kp[k0 + tid] : -1;
+      ss[tid] = (k0 + tid < K) ? ks[k0 + tid] : -1;
+    }
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < (GT * GK) / 256; q++) {
       const int e = tid + 256 * q;
       const int r = e / GK, kk = e % GK;
-      const int row = row0 + r, k = k0 + kk;
-      As[kk][r] = (row < N && k < Nh) ? W[(int64_t)row * N + ps[kk]] : 0.0;
+      As[kk][r] = (rs[r] >= 0 && ps[kk] >= 0) ? W[(int64_t)rs[r] * N + ps[kk]] : 0.0;
       const int kb = e / GT, c = e % GT;
-      const int col = col0 + c, kr = k0 + kb;
-      Bs[kb][c] = (col < Nh && kr < Nh) ? Bm[(int64_t)kr * Nh + col] : 0.0;
+      const int col = col0 + c;
+      Bs[kb][c] = (col < Nh && ss[kb] >= 0) ? Bm[(int64_t)ss[kb] * Nh + col] : 0.0;
     }
     __syncthreads();
 #pragma unroll
@@ -298,10 +468,11 @@ __global__ void __launch_bounds__(256) k_dc_gemm(int64_t n, int t, int64_t tiles
     }
     __syncthreads();
   }
+  if (K == 0) __syncthreads();          // rs written
 #pragma unroll
   for (int p = 0; p < 4; p++) {
-    const int row = row0 + ty * 4 + p;
-    if (row >= N) continue;
+    const int row = rs[ty * 4 + p];
+    if (row < 0) continue;
 #pragma unroll
     for (int q = 0; q < 4; q++) {
       const int col = col0 + tx * 4 + q;
@@ -366,12 +537,34 @@ dpr1_status dpr1_tridiag_eig(int64_t n, const double* a, const double* b, double
     if (s != DPR1_OK) return s;
     k_dc_status<<<1, 1, 0, st>>>((const unsigned*)w.bws, w.status);
     if (t > 0 || Qt) {
+      // the lists live in arrays of the batched workspace that are free once its call is done
+      Ws bw;
+      ws_layout2(n, P, true, &bw, (char*)w.bws);
+      DcAct act;
+      act.rowsrc = bw.list;
+      act.rows = bw.zlist;
+      act.inv = bw.flag;
+      act.ks = (int*)bw.fixinfo;                       // 24 n bytes: ks, kp and cnt (3 P < 3 n)
+      act.kp = act.ks + n;
+      act.cnt = act.kp + n;
+      act.call = w.status;
+      k_dc_rowsrc<<<(int)eg, 256, 0, st>>>(n, t, bw, w.pos, act);
       const int64_t Nmax = (n + P - 1) / P;            // node sizes are floor or ceil of n / 2^t
-      const int64_t Nh = (Nmax + 1) / 2;
-      const int64_t tpn = ((Nmax + GT - 1) / GT) * 2 * ((Nh + GT - 1) / GT);
-      const int64_t grid = P * tpn;
-      if (grid > 0x7fffffffLL) return DPR1_ERR_ARG;
-      k_dc_gemm<<<(unsigned)grid, 256, 0, st>>>(n, t, tpn, w.WT, w.pos, QTc, t == 0 ? Qt : QTt, ldq);
+      const int lt = Nmax >= 1024 ? 1024 : (int)((Nmax + 31) & ~(int64_t)31);
+      k_dc_lists<<<(unsigned)(P < sms * 32 ? P : sms * 32), lt, 0, st>>>(n, t, bw, w.pos, act);
+      int64_t rg = (n + 7) / 8;                        // a warp per row
+      if (rg > sms * 16) rg = sms * 16;
+      if (!Qt) {
+        const int64_t tpn = (Nmax + 31) / 32;
+        k_dc_edges<<<(unsigned)(P * tpn), 64, 0, st>>>(n, t, tpn, w.WT, QTc, QTt, act);
+      } else {
+        k_dc_copy<<<(unsigned)rg, 256, 0, st>>>(n, t, QTc, t == 0 ? Qt : QTt, ldq, act);
+        const int64_t Nh = (Nmax + 1) / 2;
+        const int64_t tpn = ((Nmax + GT - 1) / GT) * 2 * ((Nh + GT - 1) / GT);
+        const int64_t grid = P * tpn;
+        if (grid > 0x7fffffffLL) return DPR1_ERR_ARG;
+        k_dc_gemm<<<(unsigned)grid, 256, 0, st>>>(n, t, tpn, w.WT, QTc, t == 0 ? Qt : QTt, ldq, act);
+      }
       if (cudaGetLastError() != cudaSuccess) return DPR1_ERR_CUDA;
     }
     if (t > 0) {
