@@ -604,7 +604,8 @@ __global__ void __launch_bounds__(256, MINB)
             if (st != 1u) continue;
             sr = __shfl_sync(gm, sr, 0, 32);
             mr = __shfl_sync(gm, mr, 0, 32);
-            tail_row(w.dr, w.zr, n, sr, mr, pb.Vt + (int64_t)r * pb.ldv0, lane, w.vrow + 4 * (int64_t)r);
+            tail_row(w.dr, w.zr, n, sr, mr, pb.Vt + p_vbase(pb, 0) + (int64_t)r * p_ld(pb, 0), lane,
+                     w.vrow + 4 * (int64_t)r);
             if (lane == 0) {
               w.vstate[r] = 2u;
               atomicAdd(&w.counters[C_TAILROWS], 1u);
