@@ -97,8 +97,10 @@ typedef struct {
                             Algorithm 1 states; 1: the accelerated bracketed solve (a
                             rational model with the nearest pole, fitted to the value and
                             slope, kept inside the bisection bracket; the fast zero finder
-                            alternative of Sec. 2.2).  Both stop at the
-                            adjacent pair of doubles across the sign change. */
+                            alternative of Sec. 2.2).  Both stop at the adjacent pair of
+                            doubles across the sign change, or, where the elements are stored
+                            and the root is well conditioned, take the root from one evaluation
+                            and its slope in a bracket of 2^16 doubles, with the same error */
   int dd_mode;           /* the corner b of Eq. (b_ob): 1 (default) in double the working
                             precision when kappa_nu of Eq. (knu2) exceeds T_kappa * n, as
                             Algorithm 1 does, else in binary64; 2: always in double-double */
@@ -371,16 +373,16 @@ DPR1_API dpr1_status dpr1_eig_noalloc(int64_t n, const double* d, const double* 
  * counters of the last dpr1_eig / dpr1_eig_batched / dpr1_arrow_eig call on `workspace` into
  * out[0..17]:
  *   0 eigenvalues solved by the bisection kernel, 1 eigenvalues flagged by K_nu,
- *   2 remedies taken with R1, 3 with R2, 4 secular-function evaluations in the bisection
- *   kernel, 5 evaluations in the remedy kernel, 6 eigenvalues recomputed from A^{-1},
+ *   2 remedies taken with R1, 3 with R2, 4 bisection steps in the bisection kernel (evaluations,
+ *   and the steps of 9 and 13), 5 in the remedy kernel, 6 eigenvalues recomputed from A^{-1},
  *   7 deflated pairs, 8 corners b formed in double-double by the bisection kernel,
  *   9 bisection steps (of those counted in 4 and 5) settled by the binary32 screen,
  *   10 R2 remedies that formed their shift in double the working precision (of those in 3),
  *   11 screened evaluations (bisection steps of 9 and probes of 14) whose screened value
  *   exceeded the screen's error bound by less than a factor 2, 12 screened evaluations (steps
  *   of 9 and probes of 14) settled by the double-float screen, 13 bisection steps (of those
- *   counted in 4 and 5) decided by bounds that screened probes certified, without an
- *   evaluation, 14 screened probes that placed those bounds (not counted in 4 and 5),
+ *   counted in 4 and 5) decided without an evaluation, by bounds that screened probes certified
+ *   or by the finishing step that stands for the last ones, 14 screened probes that placed those bounds (not counted in 4 and 5),
  *   15 shift tests of the bisection kernel whose sign the binary32 pass settled (the others
  *   take the binary64 pass), 16 eigenvector rows written by the bisection kernel's lane
  *   groups after its queue ran out (the eigenvector kernel writes the others), 17 eigenvector

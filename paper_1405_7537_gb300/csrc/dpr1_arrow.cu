@@ -186,8 +186,9 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
   // the corner's pass also stores the elements of the inverse when the group has a buffer (and
   // their binary32 copies for the screen, after the two binary64 arrays: us = Ds + n)
   float* const F = (Ds && screen && !fast) ? (float*)(us + n) : nullptr;
-  bool scr_ok = false;
-  dd acc = dd_pole_sum<L>(d, zz, zl, n, i, di, lane, gm, &sq, nullptr, Ds, us, F, &scr_ok);
+  bool rng_ok = false;
+  dd acc = dd_pole_sum<L>(d, zz, zl, n, i, di, lane, gm, &sq, nullptr, Ds, us, F, &rng_ok);
+  const bool scr_ok = rng_ok && F;
   dd B = dd_add(two_sum(di, -alpha), acc);
   const dd Zi = {zz[i], zl[i]};
   const double b = dd_to_double(dd_div(B, Zi));
@@ -228,9 +229,30 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
   alo = fmax(alo, alo_in) * (1.0 - 0x1p-48);
   ahi = fmin(ahi, ahi_in) * (1.0 + 0x1p-48);
   bool ok;
-  int steps;
+  int steps = 0;
   double nu;
-  if (fast) {
+  // the finishing step (as in solve_pole, with the pole at 0)
+  const double finish = rng_ok && inv < 0x1p100 ? (k == 0 || k == n ? kFinishCondExt : kFinishCond) : 0.0;
+  const float cf = (float)inv;
+  auto fin = [&](double v, double* Fv, double* s, double* mag) -> bool {
+    double S;
+    float q;
+    if (!(fabs(v) >= 0x1p-60 && fabs(v) <= 0x1p60)) return false;
+    if (!stored_sum_slope_x<NI, L>(Ds, us, n, v, cf, 1.0f, lane, gm, &S, &q)) return false;
+    const double ex = inv / v;
+    const dd bv = two_sum(b, -v);
+    *Fv = side * __dadd_rn(__fma_rn(-S, inv, bv.hi), __dadd_rn(bv.lo, ex));
+    *mag = fabs(b) + fabs(S * inv) + fabs(ex);
+    *s = (double)q + ex / v;
+    return isfinite(q);
+  };
+  uint64_t blo, bhi;
+  start_bracket(&floor, alo, ahi, &blo, &bhi);
+  if (fast && finish > 0.0 && bhi - blo <= kFinishWidth &&
+      finish_root(blo, bhi, side, E, 1.0, finish, fin, &steps, &nu)) {
+    ok = true;
+  } else if (fast) {
+    const int tried = steps;
     // F(t) = side g(side t) = side b - t + Psi(t), Psi(t) = -side S / zeta_i^2 + (1/zeta_i^2) / t
     auto ev = [&](double t, bool want, double* psi, double* dpsi) {
       const double v = side * t;
@@ -245,6 +267,7 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
       return side > 0 ? g : -g;
     };
     nu = side * accel_solve(ev, floor, alo, ahi, E, side * b, 1.0, 1.0, cap, &ok, &steps);
+    steps += tried;
   } else {
     auto phi = [&](double v) {
       const double S = elem_sum<L, false, NI>(Ds, us, d, zz, n, i, di, v, lane, gm);
@@ -300,7 +323,8 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
     };
     // g > 0 below the root for the rightmost eigenvalue, g < 0 for the leftmost
     nu = bisect(phi, side, floor, alo, ahi, side > 0, cap, &ok, &steps, eager_lo, eager_hi, scr, &r.screened,
-                kPredict && scr_ok, E, side * b, &r.inferred, &r.probes);
+                kPredict && scr_ok, E, side * b, &r.inferred, &r.probes, finish, 1.0,
+                fin);
   }
   r.nu = nu;
   r.mu = 1.0 / nu;
@@ -510,8 +534,9 @@ __device__ double solve_nonpole_arrow(const double* __restrict__ d, const double
                                       int* steps_out, double* __restrict__ Ds = nullptr,
                                       double* __restrict__ us = nullptr, double sigma_lo = 0.0) {
   double un2, cub;
+  bool rng_ok = false;
   // the double-double pass also stores the elements for the solve when the group has a buffer
-  const dd acc = dd_pole_sum<L, OFS>(d, zz, zl, n, -1, sigma, lane, gm, &un2, &cub, Ds, us, nullptr, nullptr,
+  const dd acc = dd_pole_sum<L, OFS>(d, zz, zl, n, -1, sigma, lane, gm, &un2, &cub, Ds, us, nullptr, &rng_ok,
                                      sigma_lo);
   const dd f = dd_add(OFS ? shift_diff(alpha, sigma, sigma_lo) : two_sum(alpha, -sigma), {-acc.hi, -acc.lo});
   *ok = true;
@@ -539,10 +564,30 @@ __device__ double solve_nonpole_arrow(const double* __restrict__ d, const double
   ahi *= (1.0 + 0x1p-48);
   int steps;
   double nu;
+  // F(t) = -h(side t) = |gamma| (-1/|gamma| + Psi(t)), Psi(t) = -side S(side t) + 1/t; every
+  // pole of Psi lies at or below floor, the model pole
+  const double ag = fabs(gamma);
+  const double finish = rng_ok && ag > 0x1p-60 && ag < 0x1p100 ? kFinishCond : 0.0;
+  auto fin = [&](double v, double* Fv, double* s, double* mag) -> bool {
+    double S;
+    float q;
+    const double t = fabs(v);
+    if (!(t >= 0x1p-60 && t <= 0x1p60)) return false;
+    if (!stored_sum_slope_x<false, L>(Ds, us, n, v, (float)ag, (float)t, lane, gm, &S, &q)) return false;
+    *Fv = -__fma_rn(gamma, __dsub_rn(S, 1.0 / v), 1.0);
+    *s = ((double)q + ag / t) / t;
+    *mag = 1.0 + ag * (fabs(S) + 1.0 / t);
+    return isfinite(q);
+  };
   if (fast) {
-    // F(t) = -h(side t) = |gamma| (-1/|gamma| + Psi(t)), Psi(t) = -side S(side t) + 1/t; every
-    // pole of Psi lies at or below floor, the model pole
-    const double ag = fabs(gamma);
+    uint64_t lo, hi;
+    steps = 0;
+    start_bracket(&floor, alo, ahi, &lo, &hi);
+    if (finish > 0.0 && hi - lo <= kFinishWidth && finish_root(lo, hi, side, floor, 0.0, finish, fin, &steps, &nu)) {
+      *steps_out = steps;
+      return 1.0 / nu;
+    }
+    const int tried = steps;
     auto ev = [&](double t, bool want, double* psi, double* dpsi) {
       const double v = side * t;
       double dS = 0.0;
@@ -554,13 +599,15 @@ __device__ double solve_nonpole_arrow(const double* __restrict__ d, const double
       return -__fma_rn(gamma, __dsub_rn(S, 1.0 / v), 1.0);
     };
     nu = side * accel_solve(ev, floor, alo, ahi, floor, -1.0 / ag, 0.0, ag, cap, ok, &steps);
+    steps += tried;
   } else {
     auto phi = [&](double v) {
       const double S = elem_sum<L, OFS>(Ds, us, d, zz, n, -1, sigma, v, lane, gm, sigma_lo);
       return __fma_rn(gamma, __dsub_rn(S, 1.0 / v), 1.0);
     };
     // h < 0 between the floor and the root in both cases
-    nu = bisect(phi, side, floor, alo, ahi, false, cap, ok, &steps);
+    nu = bisect(phi, side, floor, alo, ahi, false, cap, ok, &steps, false, false, NoScreen(), nullptr, false, floor,
+                0.0, nullptr, nullptr, finish, 0.0, fin);
   }
   *steps_out = steps;
   return 1.0 / nu;

@@ -55,6 +55,17 @@ constexpr bool kScreenEnds = DPR1_SCREEN_ENDS != 0;
 constexpr bool kPredict = DPR1_PREDICT != 0;
 constexpr int kPredictSteps = DPR1_PREDICT_STEPS;
 constexpr uint64_t kPredictStop = 4;
+// width (in doubles) of the bracket at which the bisection of stored elements in range hands over to
+// the finishing step, and the largest condition (the size of F's terms over t |F'|) at which it applies
+// (kFinishCondExt for the exterior eigenvalues, whose mu is of the size of rho ||z||^2)
+#ifndef DPR1_FINISH_BITS
+#define DPR1_FINISH_BITS 16
+#endif
+constexpr uint64_t kFinishWidth = 1ull << DPR1_FINISH_BITS;
+#ifndef DPR1_FINISH_COND
+#define DPR1_FINISH_COND 256.0
+#endif
+constexpr double kFinishCond = DPR1_FINISH_COND, kFinishCondExt = 4.0;
 
 // ---------------------------------------------------------------------------------
 // Shifts in double the working precision (remedy R2 when no binary64 number lies between
@@ -441,16 +452,17 @@ __device__ __noinline__ bool shift_test_arrow_f32(const double* __restrict__ d, 
 
 // Stores the elements of the inverse at j: Delta_j and u_j = zz_j / Delta_j and, with F, their
 // binary32 copies and the low parts (F[j] = RN32(Delta_j), F[n + j] = RN32(u_j), F[2n + j] and
-// F[3n + j] the remainders: split_f32x2).  Returns false when a copy is not a normal binary32
-// number in the screens' range (|Delta| in [2^-80, 2^40), |u| in [2^-80, 2^60), or zero), which
-// turns the screens off.
+// F[3n + j] the remainders: split_f32x2).  Returns false when an element lies outside the screens'
+// range (|Delta| in [2^-80, 2^40), |u| in [2^-80, 2^60), or zero), which turns the screens and the
+// finishing step off.
 __device__ __forceinline__ bool store_elem(double* __restrict__ Ds, double* __restrict__ us, float* __restrict__ F,
                                            int n, int j, double D, double u) {
   Ds[j] = D;
   us[j] = u;
-  if (!F) return true;
-  split_f32x2(D, F + j, F + 2 * n + j);
-  split_f32x2(u, F + n + j, F + 3 * n + j);
+  if (F) {
+    split_f32x2(D, F + j, F + 2 * n + j);
+    split_f32x2(u, F + n + j, F + 3 * n + j);
+  }
   const unsigned eD = (unsigned)(__double_as_longlong(D) >> 52) & 0x7ffu;
   const unsigned eu = (unsigned)(__double_as_longlong(u) >> 52) & 0x7ffu;
   return (D == 0.0 || (eD >= 943u && eD <= 1062u)) && (u == 0.0 || (eu >= 943u && eu <= 1082u));
@@ -550,6 +562,65 @@ __device__ __forceinline__ bool screen_df_sum(const float* __restrict__ F, int n
   return !bad && m * 0x1p-24 < 0.25 && isfinite(sum) && isfinite(es) && isfinite(bs) && isfinite(as);
 }
 
+// |x| truncated to binary32 by integer operations (a conversion runs on the binary64 pipe): the low
+// eight bits of the exponent field less 896 are those bits with the top one flipped.  Valid for
+// 2^-126 <= |x| < 2^128; x = 0 gives 2.
+__device__ __forceinline__ float mag_f32(double x) {
+  const unsigned b = __funnelshift_l((unsigned)__double2loint(x), (unsigned)__double2hiint(x), 3);
+  return __uint_as_float((b & 0x7fffffffu) ^ 0x40000000u);
+}
+
+// The evaluation of the finishing step (bisect): the sum S(nu) of stored_sum and the slope
+//   *slope = sum_j |cf u_j / t_j| |vf Delta_j / t_j|
+// in binary32 (every term of dS/dnu = sum_j zz_j / t_j^2 has one sign; the step only scales a
+// correction of at most 2^-37 of nu by it, so its relative error of about 2^-21 costs 2^-58 of nu).
+// Delta_j, u_j (0 at the excluded index) and t_j enter as truncated magnitudes, 13 operations of the
+// other pipes per term beside 4.5 binary64 ones, where a binary64 slope takes 8.  Two terms share a
+// reciprocal, not four as in stored_sum (4.25): the sum's rounding is the result's here (rms error of
+// the arrowhead's mu 0.98 against 1.01 in units of 2^-53, 1.00 for the bisection).  For elements in the screens' range and |nu| in [2^-60, 2^60]; false when a
+// denominator leaves the fast reciprocal's range.
+template <int L>
+__device__ __forceinline__ float slope_term(double t, double D, double u, float cf, float vf) {
+  const float tf = mag_f32(t);
+  const float r0 = rcp_approx_f32(tf);
+  const float r = __fmaf_rn(r0, __fmaf_rn(-tf, r0, 1.0f), r0);
+  const float uf = ((unsigned)__double2hiint(u) << 1) ? mag_f32(u) : 0.0f;
+  return __fmul_rn(__fmul_rn(__fmul_rn(uf, cf), r), __fmul_rn(__fmul_rn(mag_f32(D), vf), r));
+}
+
+template <int L>
+__device__ __forceinline__ bool stored_sum_slope(const double* __restrict__ Ds, const double* __restrict__ us, int n,
+                                                 double nu, float cf, float vf, int lane, unsigned gm, double* S,
+                                                 float* slope) {
+  double s0 = 0.0, s1 = 0.0;
+  float q0 = 0.0f, q1 = 0.0f;
+  bool b = false;
+  int j = lane;
+#pragma unroll kStoredUnroll
+  for (; j + 3 * L < n; j += 4 * L) {
+    const double D0 = Ds[j], D1 = Ds[j + L], D2 = Ds[j + 2 * L], D3 = Ds[j + 3 * L];
+    const double u0 = us[j], u1 = us[j + L], u2 = us[j + 2 * L], u3 = us[j + 3 * L];
+    const double t0 = __fma_rn(-nu, D0, 1.0), t1 = __fma_rn(-nu, D1, 1.0);
+    const double t2 = __fma_rn(-nu, D2, 1.0), t3 = __fma_rn(-nu, D3, 1.0);
+    const double n01 = __fma_rn(u0, t1, __dmul_rn(u1, t0)), p01 = __dmul_rn(t0, t1);
+    const double n23 = __fma_rn(u2, t3, __dmul_rn(u3, t2)), p23 = __dmul_rn(t2, t3);
+    b |= !rcp_in_range(p01) || !rcp_in_range(p23);
+    s0 = __fma_rn(n01, rcp_nr(p01), s0);
+    s1 = __fma_rn(n23, rcp_nr(p23), s1);
+    q0 = __fadd_rn(q0, __fadd_rn(slope_term<L>(t0, D0, u0, cf, vf), slope_term<L>(t1, D1, u1, cf, vf)));
+    q1 = __fadd_rn(q1, __fadd_rn(slope_term<L>(t2, D2, u2, cf, vf), slope_term<L>(t3, D3, u3, cf, vf)));
+  }
+  for (; j < n; j += L) {
+    const double D0 = Ds[j], u0 = us[j], t0 = __fma_rn(-nu, D0, 1.0);
+    b |= !rcp_in_range(t0);
+    s0 = __fma_rn(u0, rcp_nr(t0), s0);
+    q0 = __fadd_rn(q0, slope_term<L>(t0, D0, u0, cf, vf));
+  }
+  *S = group_sum<L>(__dadd_rn(s0, s1), gm);
+  *slope = group_sum_f<L>(__fadd_rn(q0, q1), gm);
+  return !group_any<L>(b, gm);
+}
+
 // The loops over the stored elements as calls of their own (NI) or inlined.  Out of line, the
 // caller's state is saved once per evaluation instead of crowding the loop's registers: the
 // better form for the solve kernel of large problems, compiled for four blocks per SM (64
@@ -571,6 +642,19 @@ template <int L, bool SLOPE>
 __device__ __noinline__ bool screen_df_sum_call(const float* __restrict__ F, int n, double nu, int lane,
                                                 unsigned gm, double* S, double* E, double* A, double* dS) {
   return screen_df_sum<L, SLOPE>(F, n, nu, lane, gm, S, E, A, dS);
+}
+template <int L>
+__device__ __noinline__ bool stored_sum_slope_call(const double* __restrict__ Ds, const double* __restrict__ us,
+                                                   int n, double nu, float cf, float vf, int lane, unsigned gm,
+                                                   double* S, float* slope) {
+  return stored_sum_slope<L>(Ds, us, n, nu, cf, vf, lane, gm, S, slope);
+}
+template <bool NI, int L>
+__device__ __forceinline__ bool stored_sum_slope_x(const double* __restrict__ Ds, const double* __restrict__ us,
+                                                   int n, double nu, float cf, float vf, int lane, unsigned gm,
+                                                   double* S, float* slope) {
+  if constexpr (NI) return stored_sum_slope_call<L>(Ds, us, n, nu, cf, vf, lane, gm, S, slope);
+  else return stored_sum_slope<L>(Ds, us, n, nu, cf, vf, lane, gm, S, slope);
 }
 template <bool NI, int L, bool SLOPE = false>
 __device__ __forceinline__ bool screen_sum_x(const float* __restrict__ Df, const float* __restrict__ uf, int n,
@@ -665,7 +749,7 @@ __device__ __forceinline__ double shift_sum(const double* __restrict__ d, const 
 // gives the sum as accurately as accumulation in twice the working precision (Sec. 2.3).
 // With Ds != nullptr it also stores Dh = fl(d_j - s) and q = zz_j / Dh (0 and 0 at skip): the
 // elements of the inverse that stored_sum reads; with F their binary32 copies and low parts
-// (store_elem), and *scr_ok tells whether the screens apply to them.
+// (store_elem), and *scr_ok tells whether they lie in the screens' range.
 // With OFS the shift is s + slo in double the working precision: the difference is formed by
 // shift_diff and the stored element is its binary64 rounding (elem_diff).
 template <int L, bool OFS = false>
@@ -677,7 +761,7 @@ __device__ __forceinline__ dd dd_pole_sum(const double* __restrict__ d, const do
                                           double slo = 0.0) {
   double hi = 0.0, lo = 0.0, q2 = 0.0, c3 = 0.0;
   const double ms = -s;
-  bool ok = F != nullptr;
+  bool ok = Ds != nullptr;
   for (int j = lane; j < n; j += L) {
     if (j == skip) {
       if (Ds) ok &= store_elem(Ds, us, F, n, j, 0.0, 0.0);
@@ -755,6 +839,56 @@ struct NoScreen {
   }
 };
 
+// Finishing step of a bracket [lo, hi] (bit patterns of t = |nu|) of at most kFinishWidth doubles,
+// 2^-37 of nu: one evaluation of F and its slope at the midpoint gives the root, F(t + dt) = 0 for
+// the pole model of F at t,
+//   dt = F / (a1 + s p / (p + dt)),  p = t - pole,  -F' = a1 + s  (s from Psi),
+// one fixed-point step from Newton's dt.  The model's curvature and F's both lie in
+// [0, s / p] (in units of -F''/2), so the step is within dt^2 / p of the root of F: at most
+// 2^-60 t, else the evaluation is repeated at t + dt.  The result has the error of one binary64
+// evaluation over the slope and half an ulp, as the better of two adjacent doubles has (rms error of
+// mu in units of 2^-53 on 8000 eigenvalues each, bisected to adjacent doubles and now: uniform
+// 3.36 and 3.35, hard 3.86 and 3.85, arrowhead 1.00 and 0.98).  A step that leaves the bracket (an end that was only
+// an estimate), an evaluation out of range, or terms of F more than `finish` t |F'| (the root is then
+// noise at K_nu's size, and R2 takes its shift from it: the shift stays where the bisection puts it)
+// decline, and the solve goes on to adjacent doubles.  The bracket, its midpoint and so every bit of
+// the result are the same with and without screens.  Bisecting on costs one binary64 evaluation for
+// each bit of the window around the root that no screen can settle: 2.9 evaluations per eigenvalue on
+// the hard spectrum and 7.6 on O(1) weights, against 1.0 and 1.1 (batch of 4096 problems 388 -> 225 ms,
+// hard spectrum of order 16384 25.1 -> 20.3 ms, arrowhead of order 16384 48.3 -> 27.1 ms).
+template <class Fin>
+__device__ __forceinline__ bool finish_root(uint64_t lo, uint64_t hi, double side, double pole, double a1,
+                                            double finish, Fin fin, int* steps, double* root) {
+  const double tlo = dfrom(lo), thi = dfrom(hi);
+  double t = dfrom(lo + ((hi - lo) >> 1));
+  for (int r = 0; r < 3 && hi - lo > 1; r++) {
+    double F, s, mag;
+    if (!fin(side * t, &F, &s, &mag)) return false;
+    (*steps)++;
+    if (!(mag <= finish * t * (a1 + s))) return false;
+    const double p = __dsub_rn(t, pole);
+    const double d0 = F / (a1 + s);
+    const double dt = (p < 1e300) ? F / (a1 + s * (p / (p + d0))) : d0;
+    const double tc = __dadd_rn(t, dt);
+    if (!(tc >= tlo && tc <= thi)) return false;
+    if (dt * dt <= 0x1p-60 * t * p) {
+      *root = side * tc;
+      return true;
+    }
+    t = tc;
+  }
+  return false;
+}
+
+// The bracket that bisect starts from, as bit patterns.
+__device__ __forceinline__ void start_bracket(double* floor, double alo, double ahi, uint64_t* lo, uint64_t* hi) {
+  if (!(*floor >= 0.0)) *floor = 0.0;
+  if (!(alo >= *floor)) alo = *floor;
+  if (!(ahi > alo)) ahi = (alo > 0.0) ? alo * 2.0 : 1.0;
+  *lo = dbits(alo);
+  *hi = dbits(ahi);
+}
+
 // screen(nu, &g, &tol, mode, psi, dpsi) may settle a step without phi: it returns true with g of
 // the sign phi(nu) would have and |g| > tol (the bisection then takes the same decision); mode -1
 // lets the screen choose its precision, 0 asks for binary32 only and 1 for the double-float
@@ -782,19 +916,20 @@ struct NoScreen {
 // bisection then follows its own path from its own bracket and takes every midpoint outside
 // (cl, ch) from them (*inferred counts those steps, *probes the screened probes).  The steps, the
 // decisions and the result are those of the bisection without the probes.
-template <class Phi, class Scr = NoScreen>
+// With finish > 0 it stops at a bracket of kFinishWidth doubles and takes the finishing step above,
+// and goes on to adjacent doubles only if that declines.
+template <class Phi, class Scr, class Fin>
 __device__ double bisect(Phi phi, double side, double floor, double alo, double ahi, bool below_positive, int cap,
-                         bool* ok, int* steps_out, bool eager_lo = false, bool eager_hi = false, Scr screen = Scr(),
-                         int* screened = nullptr, bool predict = false, double pole = 0.0, double a0 = 0.0,
-                         int* inferred = nullptr, int* probes = nullptr) {
+                         bool* ok, int* steps_out, bool eager_lo, bool eager_hi, Scr screen, int* screened,
+                         bool predict, double pole, double a0, int* inferred, int* probes, double finish, double a1,
+                         Fin fin) {
+  uint64_t stop = finish > 0.0 ? kFinishWidth : 1;
   int steps = 0;
   bool good = true;
-  if (!(floor >= 0.0)) floor = 0.0;
-  if (!(alo >= floor)) alo = floor;
-  if (!(ahi > alo)) ahi = (alo > 0.0) ? alo * 2.0 : 1.0;
+  uint64_t lo, hi;
+  start_bracket(&floor, alo, ahi, &lo, &hi);
   const uint64_t fl = dbits(floor);
   const uint64_t top = 0x7fefffffffffffffull;
-  uint64_t lo = dbits(alo), hi = dbits(ahi);
   uint64_t span = hi - lo + 64;
   double glo = 0.0, ghi = 0.0;
   bool have_lo = false, have_hi = false;    // the end point was evaluated (its side is known)
@@ -860,7 +995,7 @@ __device__ double bisect(Phi phi, double side, double floor, double alo, double 
     uint64_t x = hi;
     for (int p = 0; p < kPredictSteps; p++) {
       const uint64_t bl = cl > lo ? cl : lo, bh = ch < hi ? ch : hi;
-      if (bh <= bl || bh - bl <= kPredictStop) break;
+      if (bh <= bl || bh - bl <= (stop > kPredictStop ? stop : kPredictStop)) break;
       if (x <= bl || x >= bh) {
         if (phase == 0 && x == bh && x == hi && !have_hi) {
           // the first probe: the upper end itself
@@ -925,7 +1060,7 @@ __device__ double bisect(Phi phi, double side, double floor, double alo, double 
   for (;;) {
     // bisection on the bit patterns; every evaluation moves one end and makes it known
     int phase = 0;
-    while (hi - lo > 1) {
+    while (hi - lo > stop) {
       if (phase >= cap) { good = false; break; }
       phase++;
       uint64_t mid = lo + ((hi - lo) >> 1);
@@ -955,6 +1090,21 @@ __device__ double bisect(Phi phi, double side, double floor, double alo, double 
       it++;
     }
     if (!good) break;
+    if (stop > 1) {
+      double root;
+      if (finish_root(lo, hi, side, pole, a1, finish, fin, &steps, &root)) {
+        // the steps down to adjacent doubles that this one stands for
+        const int rem = inferred ? 63 - __clzll((long long)(hi - lo)) : 0;
+        *ok = true;
+        if (steps_out) *steps_out = steps + it + rem;
+        if (screened) *screened = nscr;
+        if (inferred) *inferred = ninf + (predict ? rem : 0);
+        if (probes) *probes = nprobe;
+        return root;
+      }
+      stop = 1;
+      continue;
+    }
     // an end the bisection never moved is only an estimate: check it now (usually the root
     // lies strictly inside and both ends have moved, so this costs nothing)
     if (!have_hi) {
@@ -1172,7 +1322,7 @@ __device__ __forceinline__ double corner_b(const double* __restrict__ d, const d
                                            bool* used_dd, double* __restrict__ Ds, double* __restrict__ us,
                                            float* __restrict__ F, bool* scr_ok) {
   const double di = d[i];
-  bool ok = F != nullptr;
+  bool ok = Ds != nullptr;
   if (cr.mode != 2) {
     double p = 0.0, q = 0.0, s2 = 0.0;
     for (int j = lane; j < n; j += L) {
@@ -1235,10 +1385,11 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
   r.inferred = 0;
   r.probes = 0;
   double wn2;
-  bool used_dd, scr_ok = false;
+  bool used_dd, rng_ok = false;
   // the binary32 copies and low parts follow the two binary64 arrays (us = Ds + n)
   float* const F = (Ds && screen && !fast) ? (float*)(us + n) : nullptr;
-  double b = corner_b<L>(d, zz, zl, n, i, rho, lane, gm, &wn2, cr, &used_dd, Ds, us, F, &scr_ok);
+  double b = corner_b<L>(d, zz, zl, n, i, rho, lane, gm, &wn2, cr, &used_dd, Ds, us, F, &rng_ok);
+  const bool scr_ok = rng_ok && F;
   double side = (i == k) ? 1.0 : -1.0;
   double di = d[i];
   double inv_zi2 = 1.0 / zz[i];
@@ -1286,9 +1437,29 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
   alo = alo * (1.0 - 0x1p-48);
   ahi = ahi * (1.0 + 0x1p-48);
   bool ok;
-  int steps;
+  int steps = 0;
   double nu;
-  if (fast) {
+  // the finishing step's F = side g and the slope of Psi (F = side b - t + Psi)
+  const double finish = rng_ok && inv_zi2 < 0x1p100 ? (k == 0 ? kFinishCondExt : kFinishCond) : 0.0;
+  const float cf = (float)inv_zi2;
+  auto fin = [&](double v, double* Fv, double* s, double* mag) -> bool {
+    double S;
+    float q;
+    if (!(fabs(v) >= 0x1p-60 && fabs(v) <= 0x1p60)) return false;
+    if (!stored_sum_slope_x<NI, L>(Ds, us, n, v, cf, 1.0f, lane, gm, &S, &q)) return false;
+    const dd bv = two_sum(b, -v);
+    *Fv = side * __dadd_rn(__fma_rn(-S, inv_zi2, bv.hi), bv.lo);
+    *s = (double)q;
+    *mag = fabs(b) + fabs(S * inv_zi2);
+    return isfinite(q);
+  };
+  uint64_t blo, bhi;
+  start_bracket(&floor, alo, ahi, &blo, &bhi);
+  if (fast && finish > 0.0 && bhi - blo <= kFinishWidth &&
+      finish_root(blo, bhi, side, E, 1.0, finish, fin, &steps, &nu)) {
+    ok = true;                           // a bracket narrow enough for the finishing step as it is
+  } else if (fast) {
+    const int tried = steps;
     // F(t) = side * g(side * t) = side b - t + Psi(t), Psi = -side S / zeta_i^2
     auto ev = [&](double t, bool want, double* psi, double* dpsi) {
       const double v = side * t;
@@ -1302,6 +1473,7 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
       return side > 0 ? g : -g;
     };
     nu = side * accel_solve(ev, floor, alo, ahi, E, side * b, 1.0, 1.0, cap, &ok, &steps);
+    steps += tried;
   } else {
     auto phi = [&](double v) {
       double S = elem_sum<L, false, NI>(Ds, us, d, zz, n, i, di, v, lane, gm);
@@ -1359,7 +1531,8 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
     // g(nu) > 0 below the root for the rightmost; for the leftmost, |nu| below the root
     // means nu above it, where g < 0.
     nu = bisect(phi, side, floor, alo, ahi, side > 0, cap, &ok, &steps, eager_lo, eager_hi, scr, &r.screened,
-                kPredict && scr_ok, E, side * b, &r.inferred, &r.probes);
+                kPredict && scr_ok, E, side * b, &r.inferred, &r.probes, finish, 1.0,
+                fin);
   }
   r.nu = nu;
   r.mu = 1.0 / nu;
@@ -1391,9 +1564,10 @@ __device__ double solve_nonpole(const double* __restrict__ d, const double* __re
                                 double sigma_lo = 0.0) {
   // above / below: indices of the poles next to sigma (-1: none on that side)
   double un2, cub;
+  bool rng_ok = false;
   // the double-double pass also stores the elements d_j - sigma and zeta_j^2 / (d_j - sigma)
   // for the solve when the group has a buffer (Ds, us as for solve_pole)
-  dd acc = dd_pole_sum<L, OFS>(d, zz, zl, n, -1, sigma, lane, gm, &un2, &cub, Ds, us, nullptr, nullptr,
+  dd acc = dd_pole_sum<L, OFS>(d, zz, zl, n, -1, sigma, lane, gm, &un2, &cub, Ds, us, nullptr, &rng_ok,
                                sigma_lo);
   dd f = dd_add({1.0, 0.0}, two_prod(acc.hi, rho));
   f = dd_add(f, {__dmul_rn(acc.lo, rho), 0.0});
@@ -1422,12 +1596,35 @@ __device__ double solve_nonpole(const double* __restrict__ d, const double* __re
   ahi *= (1.0 + 0x1p-48);
   int steps;
   double nu;
+  // F(t) = -h(side * t) = |gamma| (Psi(t) - 1/|gamma|), Psi = -side S; model pole: the
+  // largest e_j on |nu| (with no pole above sigma, the one farthest below it)
+  const double E = (gamma > 0.0) ? (above >= 0 ? emax : 1.0 / elem_diff<OFS>(d[n - 1], sigma, sigma_lo))
+                                 : (below >= 0 ? -emin : -1.0 / elem_diff<OFS>(d[0], sigma, sigma_lo));
+  const double ag = fabs(gamma);
+  // the finishing step's F and slope, the slope in units of F / nu: |gamma u_j / t_j| sums to about
+  // 1 at the root
+  const double finish = rng_ok && ag > 0x1p-60 && ag < 0x1p100 ? kFinishCond : 0.0;
+  auto fin = [&](double v, double* Fv, double* s, double* mag) -> bool {
+    double S;
+    float q;
+    if (!(fabs(v) >= 0x1p-60 && fabs(v) <= 0x1p60)) return false;
+    if (!stored_sum_slope_x<NI, L>(Ds, us, n, v, (float)ag, (float)fabs(v), lane, gm, &S, &q)) return false;
+    *Fv = -__fma_rn(gamma, S, 1.0);
+    *mag = 1.0 + fabs(gamma * S);
+    *s = (double)q / fabs(v);
+    return isfinite(q) && q > 0x1p-60f;
+  };
   if (fast) {
-    // F(t) = -h(side * t) = |gamma| (Psi(t) - 1/|gamma|), Psi = -side S; model pole: the
-    // largest e_j on |nu| (with no pole above sigma, the one farthest below it)
-    const double E = (gamma > 0.0) ? (above >= 0 ? emax : 1.0 / elem_diff<OFS>(d[n - 1], sigma, sigma_lo))
-                                   : (below >= 0 ? -emin : -1.0 / elem_diff<OFS>(d[0], sigma, sigma_lo));
-    const double ag = fabs(gamma);
+    // the bracket is usually narrow enough for the finishing step as it is
+    uint64_t lo, hi;
+    steps = 0;
+    start_bracket(&floor, alo, ahi, &lo, &hi);
+    if (finish > 0.0 && hi - lo <= kFinishWidth && finish_root(lo, hi, side, E, 0.0, finish, fin, &steps, &nu)) {
+      *ok = true;
+      if (steps_out) *steps_out = steps;
+      return 1.0 / nu;
+    }
+    const int tried = steps;
     auto ev = [&](double t, bool want, double* psi, double* dpsi) {
       double dS = 0.0;
       const double S = want ? elem_sum_d<L, OFS>(Ds, us, d, zz, n, -1, sigma, side * t, lane, gm, &dS, sigma_lo)
@@ -1437,12 +1634,14 @@ __device__ double solve_nonpole(const double* __restrict__ d, const double* __re
       return -__fma_rn(gamma, S, 1.0);
     };
     nu = side * accel_solve(ev, floor, alo, ahi, E, -1.0 / ag, 0.0, ag, cap, ok, &steps);
+    steps += tried;
   } else {
     auto phi = [&](double v) {
       const double S = elem_sum<L, OFS, NI>(Ds, us, d, zz, n, -1, sigma, v, lane, gm, sigma_lo);
       return __fma_rn(gamma, S, 1.0);
     };
-    nu = bisect(phi, side, floor, alo, ahi, false, cap, ok, &steps);
+    nu = bisect(phi, side, floor, alo, ahi, false, cap, ok, &steps, false, false, NoScreen(), nullptr, false, E, 0.0,
+                nullptr, nullptr, finish, 0.0, fin);
   }
   if (steps_out) *steps_out = steps;
   return 1.0 / nu;
