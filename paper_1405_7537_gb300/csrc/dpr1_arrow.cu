@@ -194,7 +194,7 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
   const double b = dd_to_double(dd_div(B, Zi));
   const double inv = 1.0 / zz[i];
   const double wn2 = sq / Zi.hi + inv;          // squared border: w_j (j != i) and 1/zeta_i
-  const double wn = sqrt(wn2);
+  const double wn = root(wn2);
   const double side = (i == k) ? 1.0 : -1.0;
   double floor, E;
   // the caller's [alo, ahi] rests on the shift test (or the 2 x 2 interlacing bounds) and is
@@ -204,25 +204,25 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
   ahi = INFINITY;
   if (side > 0) {
     // largest pole of g: the nearest pole above d_i (or, for i = 0, the farthest below), or 0
-    const double dmax = (i > 0) ? 1.0 / (d[i - 1] - di) : (n > 1 ? 1.0 / (d[n - 1] - di) : -INFINITY);
+    const double dmax = (i > 0) ? quot(1.0, d[i - 1] - di) : (n > 1 ? quot(1.0, d[n - 1] - di) : -INFINITY);
     const double pmax = fmax(dmax, 0.0);
     floor = pmax;
     E = pmax;
     alo = fmax(alo, b);
     ahi = fmin(ahi, fmax(b, pmax) + wn);
-    if (b > pmax) ahi = fmin(ahi, b + wn2 / (b - pmax));
+    if (b > pmax) ahi = fmin(ahi, b + quot(wn2, b - pmax));
     // smallest pole: the nearest delta_j below d_i (or the farthest above), or 0
-    const double dmin = (i + 1 < n) ? 1.0 / (d[i + 1] - di) : (n > 1 ? 1.0 / (d[0] - di) : INFINITY);
+    const double dmin = (i + 1 < n) ? quot(1.0, d[i + 1] - di) : (n > 1 ? quot(1.0, d[0] - di) : INFINITY);
     quad_bracket(b, fmin(dmin, 0.0), pmax, wn2, &alo, &ahi);
   } else {
-    const double dmin = (i + 1 < n) ? 1.0 / (d[i + 1] - di) : (n > 1 ? 1.0 / (d[0] - di) : INFINITY);
+    const double dmin = (i + 1 < n) ? quot(1.0, d[i + 1] - di) : (n > 1 ? quot(1.0, d[0] - di) : INFINITY);
     const double pmin = fmin(dmin, 0.0);
     floor = -pmin;
     E = -pmin;
     alo = fmax(alo, -b);
     ahi = fmin(ahi, -fmin(b, pmin) + wn);
-    if (b < pmin) ahi = fmin(ahi, -b + wn2 / (pmin - b));
-    const double dmx = (i > 0) ? 1.0 / (d[i - 1] - di) : (n > 1 ? 1.0 / (d[n - 1] - di) : -INFINITY);
+    if (b < pmin) ahi = fmin(ahi, -b + quot(wn2, pmin - b));
+    const double dmx = (i > 0) ? quot(1.0, d[i - 1] - di) : (n > 1 ? quot(1.0, d[n - 1] - di) : -INFINITY);
     quad_bracket(-b, -fmax(dmx, 0.0), -pmin, wn2, &alo, &ahi);
   }
   const bool eager_lo = alo_in > alo, eager_hi = ahi_in < ahi;
@@ -275,14 +275,12 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
     };
     // binary32 screen as in solve_pole; the extra pole's term fl(inv / v) is the same in both
     // evaluations, and the bound also covers the rounding of the intermediate difference X
-    const double mlane = (double)((n + L - 1) / L);
-    auto decide = [&](double Sx, double Ex, double aS, double v, double* g, double* tl) -> bool {
-      const double E64 = stored_sum_error<L>(mlane, aS);
-      const double X = __dsub_rn(__dsub_rn(b, v), __dmul_rn(Sx, inv));
-      const double G = __dadd_rn(X, inv / v);
-      const double tol = 1.01 * (inv * (Ex + E64 + 0x1p-51 * aS) + 0x1p-51 * fabs(X));
-      if (!(fabs(G) > tol)) return false;
-      if (fabs(G) <= 2.0 * tol) r.screened_near++;
+    auto decide = [&](const Screened& c, double v, double Sz, double ex, double* g, double* tl) -> bool {
+      const double X = __dsub_rn(__dsub_rn(b, v), Sz);
+      const double G = __dadd_rn(X, ex);
+      const double tol = __fma_rn(inv, (double)c.x, 1.01 * 0x1p-51 * fabs(X));
+      if (!mag_greater(G, tol)) return false;
+      if (!mag_greater(G, __dadd_rn(tol, tol))) r.screened_near++;
       *g = G;
       *tl = tol;
       return true;
@@ -291,12 +289,14 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
     int f32_fail = 0;
     auto scr = [&](double v, double* g, double* tl, int mode, double* psi, double* dpsi) -> bool {
       if (!scr_ok) return false;
-      double Sx, Ex, aS, dS = 0.0;
+      Screened c;
+      const double ex = inv / v;                    // phi's term, bit for bit
+      double Sz = 0.0;
       bool ok = false;
       if (mode == 0 || (mode < 0 && f32_fail < kScreen32Tries)) {
-        ok = (psi ? screen_sum_x<NI, L, true>(F, F + n, n, v, lane, gm, &Sx, &Ex, &aS, &dS)
-                  : screen_sum_x<NI, L>(F, F + n, n, v, lane, gm, &Sx, &Ex, &aS)) &&
-             decide(Sx, Ex, aS, v, g, tl);
+        c = psi ? screen_sum_x<NI, L, true>(F, F + n, n, v, lane, gm) : screen_sum_x<NI, L, false>(F, F + n, n, v, lane, gm);
+        Sz = __dmul_rn(c.S, inv);
+        ok = decide(c, v, Sz, ex, g, tl);
         if (ok) {
           if (mode < 0) f32_fail = 0;
         } else {
@@ -306,18 +306,16 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
       }
       if (!ok) {
         if (mode == 1) f32_fail = kScreen32Tries;   // the probes have reached the binary32 window
-        ok = kScreenDf &&
-             (psi ? screen_df_sum_x<NI, L, true>(F, n, v, lane, gm, &Sx, &Ex, &aS, &dS)
-                  : screen_df_sum_x<NI, L>(F, n, v, lane, gm, &Sx, &Ex, &aS)) &&
-             decide(Sx, Ex, aS, v, g, tl);
-        if (!ok) return false;
+        if (!kScreenDf) return false;
+        c = psi ? screen_df_sum_x<NI, L, true>(F, n, v, lane, gm) : screen_df_sum_x<NI, L, false>(F, n, v, lane, gm);
+        Sz = __dmul_rn(c.S, inv);
+        if (!decide(c, v, Sz, ex, g, tl)) return false;
         r.screened_df++;
       }
       // Psi and Psi' on t = |nu| as the accelerated solve forms them (with the pole at 0)
       if (psi) {
-        const double t = fabs(v), ex = inv / t;
-        *psi = -side * __dmul_rn(Sx, inv) + ex;
-        *dpsi = -__dmul_rn(dS, inv) - ex / t;
+        *psi = -side * Sz + fabs(ex);
+        *dpsi = -__dmul_rn((double)c.slope, inv) - quot_approx(ex, v);
       }
       return true;
     };
@@ -472,9 +470,9 @@ __global__ void __launch_bounds__(256, DPR1_SOLVE_MIN_BLOCKS) k_arrow_solve(int 
       const double dk = d[k];
       const double tau = __dmul_rn(__dsub_rn(d[k - 1], dk), 0.5);
       const double c = __dsub_rn(__dsub_rn(alpha, dk), tau);
-      double sp = 0.0, sn = 0.0, F = 0.0, EF = 0.0;
-      shift32 = kArrowShift32 && screen && shift_test_arrow_f32<L>(d, zz, n, dk, tau, c, lane, gm, &F, &EF) &&
-                fabs(F) > EF;
+      double sp = 0.0, sn = 0.0, F = 0.0;
+      const int sf = (kArrowShift32 && screen) ? shift_test_arrow_f32<L>(d, zz, n, dk, tau, c, lane, gm) : 0;
+      shift32 = sf != 0;
       if (!shift32) {
         for (int j = lane; j < n; j += L) {
           const double t = __dmul_rn(zz[j], rcp(__dsub_rn(__dsub_rn(d[j], dk), tau)));
@@ -485,12 +483,12 @@ __global__ void __launch_bounds__(256, DPR1_SOLVE_MIN_BLOCKS) k_arrow_solve(int 
         sn = group_sum<L>(sn, gm);
         F = c - (sp + sn);
       }
-      alo = 1.0 / tau;
+      alo = quot(1.0, tau);
       // the upper bracket end from the binary64 pass's partial sums is left out when the
       // binary32 pass may decide (both paths then start the bisection from the same bracket):
       //   mu in (0, tau]:   zeta_k^2 nu <= sum_{j<k} zeta_j^2/((d_j - d_k) - tau) + d_k - alpha + tau
       //   mu in [-tau, 0):  zeta_{k-1}^2 |nu| <= -sum_{j>=k} zeta_j^2/((d_j - d_k) - tau) + alpha - d_{k-1} + tau
-      if (F < 0.0) {
+      if (sf != 0 ? sf < 0 : F < 0.0) {
         i = k;
         if (!kArrowShift32) ahi = (sp + (dk - alpha) + tau) / zz[k];
       } else {

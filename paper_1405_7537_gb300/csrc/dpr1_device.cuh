@@ -110,6 +110,39 @@ static __device__ __noinline__ double rcp_ieee(double x) { return 1.0 / x; }
 // 1/x within one ulp for every x (the IEEE quotient outside the fast range)
 __device__ __forceinline__ double rcp(double x) { return rcp_in_range(x) ? rcp_nr(x) : rcp_ieee(x); }
 
+// Quotients and square roots of the solves' scalar work (brackets, placed points, the finishing
+// correction), which every lane of a group computes: the IEEE operations take 10 to 15 binary64
+// instructions each, and a solve made about 1000 scalar ones per eigenvalue, as many as its sums take
+// at order 2000 with 32 lanes.  quot: a / b within 2 ulps (a times the IEEE reciprocal outside
+// rcp_nr's range); quot_approx: within 2^-38 (the seed's 2^-20 and one Newton step), NaN or infinity out
+// of range, which its callers treat as "no point".  root: sqrt(x) within 2 ulps by two Newton steps on the
+// hardware's reciprocal square root, sqrt out of line for the rest.
+__device__ __forceinline__ double quot(double a, double b) { return __dmul_rn(a, rcp(b)); }
+__device__ __forceinline__ double quot_approx(double a, double b) {
+  const double r = rcp_approx(b);
+  return __dmul_rn(a, __fma_rn(r, __fma_rn(-b, r, 1.0), r));
+}
+static __device__ __noinline__ double sqrt_ieee(double x) { return sqrt(x); }
+__device__ __forceinline__ double root(double x) {
+  if (!((unsigned)(__double2hiint(x)) - 0x03700000u < 0x78f00000u)) return sqrt_ieee(x);   // x in [2^-968, 2^967)
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double h = __dmul_rn(0.5, y);
+  double s = __dmul_rn(x, y);
+  s = __fma_rn(__fma_rn(-s, s, x), h, s);
+  return __fma_rn(__fma_rn(-s, s, x), h, s);
+}
+
+// order of the magnitudes of doubles as integers (a binary64 comparison takes the binary64 pipe):
+// |a| > |b|, false when a is NaN or infinite
+__device__ __forceinline__ bool mag_greater(double a, double b) {
+  const unsigned long long x = (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
+  const unsigned long long y = (unsigned long long)__double_as_longlong(b) & 0x7fffffffffffffffull;
+  return x > y && x < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool finite(double a) { return (__double2hiint(a) & 0x7ff00000) != 0x7ff00000; }
+__device__ __forceinline__ bool is_negative(double a) { return __double2hiint(a) < 0; }
+
 // dd / dd to about 2^-104 relative: q1 = a.hi/b.hi, then one correction digit from the
 // exact residual a.hi - q1 b.hi (fma), the low parts and the divisor's reciprocal.
 __device__ __forceinline__ dd dd_div(dd a, dd b) {

@@ -639,12 +639,11 @@ __global__ void __launch_bounds__(256, MINB)
     } else {
       double dk = d[k];
       double tau = __dmul_rn(__dsub_rn(d[k - 1], dk), 0.5);
-      double sp = 0.0, sn = 0.0, F = 0.0, EF = 0.0;
+      double sp = 0.0, sn = 0.0, F = 0.0;
       // the binary32 pass decides where its bound settles the sign (the binary64 pass's sign)
-      const bool f32 = kShift32 && screen && shift_test_f32<L>(d, zz, n, dk, tau, rho, lane, gm, &F, &EF) &&
-                       fabs(F) > EF;
-      shift32 = f32;
-      if (!f32) {
+      const int sf = (kShift32 && screen) ? shift_test_f32<L>(d, zz, n, dk, tau, rho, lane, gm) : 0;
+      shift32 = sf != 0;
+      if (sf == 0) {
         for (int j = lane; j < n; j += L) {
           double den = __dsub_rn(__dsub_rn(d[j], dk), tau);
           double t = __dmul_rn(zz[j], rcp(den));
@@ -655,9 +654,9 @@ __global__ void __launch_bounds__(256, MINB)
         sn = group_sum<L>(sn, gm);
         F = 1.0 + rho * (sp + sn);
       }
-      alo = 1.0 / tau;
+      alo = quot(1.0, tau);
       ahi = INFINITY;
-      if (F > 0.0) {
+      if (sf != 0 ? sf > 0 : F > 0.0) {
         i = k;
         if (kShiftAhi) ahi = (1.0 + rho * sp) / (rho * zz[k]);
       } else {

@@ -243,10 +243,19 @@ __device__ __forceinline__ double stored_sum(const double* __restrict__ Ds, cons
 // |nu| <= 2^60) and with |nu Delta_j / t_j| <= 2^20, so every |t_j| lies in [2^-22, 2^101) and
 // every numerator and denominator of stored_sum between 2^-160 and 2^410, inside the fast
 // reciprocal's range.
+// Returned per unit of A, with 2^-51 for the roundings of the products with 1 / zeta_i^2.
 template <int L>
-__device__ __forceinline__ double stored_sum_error(double m, double A) {
-  return (0.25 * m + 14.0 + (double)tree_roundings<L>()) * 0x1p-53 * A;
+__device__ __forceinline__ float stored_sum_error(int m) {
+  return (0.25f * (float)m + 18.01f + (float)tree_roundings<L>()) * 0x1p-53f;
 }
+
+// What a screen returns: the sum S, a bound x on |S - S64| (S64 the sum stored_sum would return, with
+// the roundings of both products with 1 / zeta_i^2; every factor rounded up by the final 1 + 2^-20, or
+// infinity when the screen does not apply) and with SLOPE an estimate of dS/dnu.
+struct Screened {
+  double S;
+  float x, slope;
+};
 
 // Binary32 screen of a bisection step.  From the binary32 copies Df_j = fl32(Delta_j) and
 // uf_j = fl32(u_j) and vf = fl32(nu) (each within eps = 2^-24 relative) each lane forms
@@ -264,13 +273,12 @@ __device__ __forceinline__ double stored_sum_error(double m, double A) {
 // the bound's own sum; the last term for results below the binary32 normal range) holds for
 // |S - sum_j T_j|, and A = 1.02 sum_j e_j / (6 eps) + E >= sum_j |T_j|.  The copies and nu
 // must lie in the ranges checked by store_elem and here (|nu| in [2^-60, 2^60], so |p| <= 2^100).
-// Returns false when the screen does not apply (a range, w, or a non-finite sum or bound).
-// With SLOPE it also returns *dS ~ dS/dnu = sum_j (u_j / t_j)(Delta_j / t_j) (no bound: the
+// The bound is infinite when the screen does not apply (a range, w, or a non-finite sum).
+// With SLOPE it also returns dS/dnu = sum_j (u_j / t_j)(Delta_j / t_j) roughly (no bound: the
 // probes of the bisection only place points with it).
-template <int L, bool SLOPE = false>
-__device__ __forceinline__ bool screen_sum(const float* __restrict__ Df, const float* __restrict__ uf, int n,
-                                           double nu, int lane, unsigned gm, double* S, double* E, double* A,
-                                           double* dS = nullptr) {
+template <int L, bool SLOPE>
+__device__ __forceinline__ Screened screen_sum(const float* __restrict__ Df, const float* __restrict__ uf, int n,
+                                               double nu, int lane, unsigned gm) {
   const float vf = __double2float_rn(nu);
   const float av = fabsf(vf);
   float sh = 0.0f, sl = 0.0f, e = 0.0f, sd = 0.0f;
@@ -294,15 +302,17 @@ __device__ __forceinline__ bool screen_sum(const float* __restrict__ Df, const f
   // stay far below eps A, inside the bound's 5% margin), the bound's sum raised by 2^-20 to cover
   // its own tree_roundings (at most 16)
   group_sum2_f<L>(&sh, &sl, gm);
-  const double sum = __dadd_rn((double)sh, (double)sl);
-  const double es = (double)group_sum_f<L>(e, gm) * (1.0 + 0x1p-20);
-  if (SLOPE) *dS = (double)group_sum_f<L>(sd, gm);
+  e = group_sum_f<L>(e, gm);
+  Screened r;
+  r.S = __dadd_rn((double)sh, (double)sl);
+  r.slope = SLOPE ? group_sum_f<L>(sd, gm) : 0.0f;
   bad = group_any<L>(bad, gm);
-  const double m = (double)((n + L - 1) / L);
-  *S = sum;
-  *E = 1.05 * (1.0 + 2.0 * (m + 2.0) * 0x1p-24) * 0x1p-24 * es + 8.0 * (double)n * 0x1p-126;
-  *A = (1.02 / 6.0) * es + *E;
-  return !bad && m * 0x1p-24 < 0.25 && isfinite(sum) && isfinite(es);
+  // x = 1.01 (E + stored_sum_error A)
+  const int m = (n + L - 1) / L;
+  const float c = 1.05f * (1.0f + 2.0f * ((float)m + 2.0f) * 0x1p-24f) * 0x1p-24f;
+  const float x = 1.01f * (1.0f + 0x1p-19f) * ((c + stored_sum_error<L>(m) * (0.1701f + c)) * e + (float)n * 0x1p-122f);
+  r.x = (!bad && m < (1 << 22) && x < INFINITY) ? x : INFINITY;
+  return r;
 }
 
 // x = hi + lo with hi = RN32(x) (the binary32 number nearest x, ties to even) and lo = x - hi
@@ -380,8 +390,8 @@ __device__ __forceinline__ float rn32(double x, bool* ok) {
 // decision on the sign of F32 with |F32| > E is the binary64 pass's decision.
 template <int L>
 __device__ __forceinline__ bool shift_sum_f32(const double* __restrict__ d, const double* __restrict__ zz, int n,
-                                              double dk, double tau, int lane, unsigned gm, double* S, double* es_out,
-                                              double* as_out) {
+                                              double dk, double tau, int lane, unsigned gm, double* S, float* es_out,
+                                              float* as_out) {
   bool ok = true;
   const float tf = rn32(tau, &ok);
   float sh = 0.0f, sl = 0.0f, e = 0.0f, a1 = 0.0f;
@@ -407,47 +417,48 @@ __device__ __forceinline__ bool shift_sum_f32(const double* __restrict__ d, cons
   // the lane group's sums in binary32 as in screen_sum
   group_sum2_f<L>(&sh, &sl, gm);
   *S = __dadd_rn((double)sh, (double)sl);
-  *es_out = (double)group_sum_f<L>(e, gm) * (1.0 + 0x1p-20);
-  *as_out = (double)group_sum_f<L>(a1, gm) * (1.0 + 0x1p-20);
+  *es_out = group_sum_f<L>(e, gm);
+  *as_out = group_sum_f<L>(a1, gm);
   return !group_any<L>(!ok, gm);
 }
 
-// D + rho z z^T: F = 1 + rho S.
+// The bound of |S32 - S| and |S64 - S| together, rounded up (the factor 1 + 2^-18 covers the roundings
+// of the bound's own sums and of this expression):
+//   E32 = 1.05 g eps es + (2 + tree) 2^-53 g as + 4 n 2^-149,
+//   E64 = 1.01 2^-53 g (es + (m + 16 + tree) as),  g = 1 + 2 (m + 2) eps,
+// and 2^-50 g as for the roundings of the last operations.
 template <int L>
-__device__ __noinline__ bool shift_test_f32(const double* __restrict__ d, const double* __restrict__ zz, int n,
-                                            double dk, double tau, double rho, int lane, unsigned gm, double* F,
-                                            double* E) {
-  double S, es, as;
+__device__ __forceinline__ float shift_bound(int n, float es, float as) {
+  const float m = (float)((n + L - 1) / L), tr = (float)tree_roundings<L>();
+  const float g = 1.0f + 2.0f * (m + 2.0f) * 0x1p-24f;
+  return 1.01f * (1.0f + 0x1p-18f) * g *
+         ((1.05f * 0x1p-24f + 1.01f * 0x1p-53f) * es + (1.01f * m + 28.0f + 2.01f * tr) * 0x1p-53f * as + (float)n * 0x1p-126f);
+}
+
+// D + rho z z^T: the sign (+1, -1) of F = 1 + rho S, 0 where the bound leaves it open.
+template <int L>
+__device__ __noinline__ int shift_test_f32(const double* __restrict__ d, const double* __restrict__ zz, int n,
+                                           double dk, double tau, double rho, int lane, unsigned gm) {
+  double S;
+  float es, as;
   const bool ok = shift_sum_f32<L>(d, zz, n, dk, tau, lane, gm, &S, &es, &as);
-  const double m = (double)((n + L - 1) / L);
-  const double g = 1.0 + 2.0 * (m + 2.0) * 0x1p-24;
-  const double F32 = 1.0 + rho * S;
-  const double E32 = rho * (1.05 * g * 0x1p-24 * es + (2.0 + tree_roundings<L>()) * 0x1p-53 * g * as +
-                            4.0 * (double)n * 0x1p-149);
-  const double E64 = 1.01 * 0x1p-53 * rho * g * (es + (m + 16.0 + tree_roundings<L>()) * as);
-  *F = F32;
-  *E = 1.01 * (E32 + E64 + 0x1p-50 * (1.0 + rho * g * as));
-  return ok && isfinite(F32) && isfinite(*E);
+  const double F = __fma_rn(rho, S, 1.0);
+  const double E = __fma_rn(rho, (double)shift_bound<L>(n, es, as), 0x1p-49);
+  return (ok && es < INFINITY && mag_greater(F, E)) ? (is_negative(F) ? -1 : 1) : 0;
 }
 
 // The arrowhead [D z; z^T alpha]: F = c - S with c = fl(fl(alpha - d_k) - tau), the value the
 // binary64 pass subtracts its sum fl(sp + sn) from; fl(c - x) has the sign of c - x, so the
 // binary64 decision is the sign of c - fl(sp + sn), within the same bound of c - S32.
 template <int L>
-__device__ __noinline__ bool shift_test_arrow_f32(const double* __restrict__ d, const double* __restrict__ zz, int n,
-                                                  double dk, double tau, double c, int lane, unsigned gm, double* F,
-                                                  double* E) {
-  double S, es, as;
+__device__ __noinline__ int shift_test_arrow_f32(const double* __restrict__ d, const double* __restrict__ zz, int n,
+                                                 double dk, double tau, double c, int lane, unsigned gm) {
+  double S;
+  float es, as;
   const bool ok = shift_sum_f32<L>(d, zz, n, dk, tau, lane, gm, &S, &es, &as);
-  const double m = (double)((n + L - 1) / L);
-  const double g = 1.0 + 2.0 * (m + 2.0) * 0x1p-24;
-  const double F32 = __dsub_rn(c, S);
-  const double E32 = 1.05 * g * 0x1p-24 * es + (2.0 + tree_roundings<L>()) * 0x1p-53 * g * as +
-                     4.0 * (double)n * 0x1p-149;
-  const double E64 = 1.01 * 0x1p-53 * g * (es + (m + 16.0 + tree_roundings<L>()) * as);
-  *F = F32;
-  *E = 1.01 * (E32 + E64 + 0x1p-50 * (fabs(c) + g * as));
-  return ok && isfinite(F32) && isfinite(*E);
+  const double F = __dsub_rn(c, S);
+  const double E = __fma_rn(0x1p-49, fabs(c), (double)shift_bound<L>(n, es, as));
+  return (ok && es < INFINITY && mag_greater(F, E)) ? (is_negative(F) ? -1 : 1) : 0;
 }
 
 // Stores the elements of the inverse at j: Delta_j and u_j = zz_j / Delta_j and, with F, their
@@ -498,12 +509,12 @@ __device__ __forceinline__ bool store_elem(double* __restrict__ Ds, double* __re
 //   E = 1.05 g (eps^2 sum e_j + eps sum bl) + g ((2 + tree_roundings) 2^-53 + 2^-140) sum |q1|
 //       + 48 n 2^-149
 // bounds |S - sum_j T_j|, and A = 1.001 g sum |q1| + E >= sum_j |T_j|.  Ranges as screen_sum
-// (w <= 2^20: |t| >= 2^-21, every |q1| below 2^82).  Returns false when the screen does not
-// apply (a range, w, or a non-finite sum or bound).
-// With SLOPE it also returns *dS as screen_sum does (from the high parts).
-template <int L, bool SLOPE = false>
-__device__ __forceinline__ bool screen_df_sum(const float* __restrict__ F, int n, double nu, int lane, unsigned gm,
-                                              double* S, double* E, double* A, double* dS = nullptr) {
+// (w <= 2^20: |t| >= 2^-21, every |q1| below 2^82).  The bound is infinite when the screen does not
+// apply (a range, w, or a non-finite sum).
+// With SLOPE it also returns the slope as screen_sum does (from the high parts).
+template <int L, bool SLOPE>
+__device__ __forceinline__ Screened screen_df_sum(const float* __restrict__ F, int n, double nu, int lane,
+                                                  unsigned gm) {
   const float* __restrict__ Dh = F;
   const float* __restrict__ uh = F + n;
   const float* __restrict__ Dl = F + 2 * n;
@@ -545,21 +556,23 @@ __device__ __forceinline__ bool screen_df_sum(const float* __restrict__ F, int n
     a1 = __fadd_rn(a1, aq);
     e = __fmaf_rn(aq, __fmaf_rn(16.0f, w, 32.0f), e);
   }
-  const double sum = group_sum<L>(__dadd_rn(__dadd_rn((double)sh, (double)sl), (double)sll), gm);
-  // the bound's sums of positive terms in binary32, raised by 2^-20 to cover their own
-  // tree_roundings (at most 16)
-  const double es = (double)group_sum_f<L>(e, gm) * (1.0 + 0x1p-20);
-  const double bs = (double)group_sum_f<L>(bl, gm) * (1.0 + 0x1p-20);
-  const double as = (double)group_sum_f<L>(a1, gm) * (1.0 + 0x1p-20);
-  if (SLOPE) *dS = (double)group_sum_f<L>(sd, gm);
+  Screened r;
+  r.S = group_sum<L>(__dadd_rn(__dadd_rn((double)sh, (double)sl), (double)sll), gm);
+  // the bound's sums of positive terms in binary32: their own tree_roundings (at most 16) lie in the
+  // final factor
+  e = group_sum_f<L>(e, gm);
+  bl = group_sum_f<L>(bl, gm);
+  a1 = group_sum_f<L>(a1, gm);
+  r.slope = SLOPE ? group_sum_f<L>(sd, gm) : 0.0f;
   bad = group_any<L>(bad, gm);
-  const double m = (double)((n + L - 1) / L);
-  const double g = 1.0 + 2.0 * (m + 2.0) * 0x1p-24;
-  *S = sum;
-  *E = 1.05 * g * (0x1p-48 * es + 0x1p-24 * bs) + g * ((2.0 + tree_roundings<L>()) * 0x1p-53 + 0x1p-140) * as +
-       48.0 * (double)n * 0x1p-149;
-  *A = 1.001 * g * as + *E;
-  return !bad && m * 0x1p-24 < 0.25 && isfinite(sum) && isfinite(es) && isfinite(bs) && isfinite(as);
+  // x = 1.01 (E + stored_sum_error A)
+  const int m = (n + L - 1) / L;
+  const float g = 1.0f + 2.0f * ((float)m + 2.0f) * 0x1p-24f;
+  const float cE = 1.0f + 0x1p-20f, cA = 1.002f * g * stored_sum_error<L>(m) + g * (2.01f + tree_roundings<L>()) * 0x1p-53f;
+  const float x = 1.01f * (1.0f + 0x1p-19f) *
+                  (1.05f * g * cE * (0x1p-48f * e + 0x1p-24f * bl) + cA * a1 + (float)n * 0x1p-126f);
+  r.x = (!bad && m < (1 << 22) && x < INFINITY) ? x : INFINITY;
+  return r;
 }
 
 // |x| truncated to binary32 by integer operations (a conversion runs on the binary64 pipe): the low
@@ -633,15 +646,14 @@ __device__ __noinline__ double stored_sum_call(const double* __restrict__ Ds, co
   return stored_sum<L, OFS>(Ds, us, d, zz, n, i, di, nu, lane, gm, dlo);
 }
 template <int L, bool SLOPE>
-__device__ __noinline__ bool screen_sum_call(const float* __restrict__ Df, const float* __restrict__ uf, int n,
-                                             double nu, int lane, unsigned gm, double* S, double* E, double* A,
-                                             double* dS) {
-  return screen_sum<L, SLOPE>(Df, uf, n, nu, lane, gm, S, E, A, dS);
+__device__ __noinline__ Screened screen_sum_call(const float* __restrict__ Df, const float* __restrict__ uf, int n,
+                                                 double nu, int lane, unsigned gm) {
+  return screen_sum<L, SLOPE>(Df, uf, n, nu, lane, gm);
 }
 template <int L, bool SLOPE>
-__device__ __noinline__ bool screen_df_sum_call(const float* __restrict__ F, int n, double nu, int lane,
-                                                unsigned gm, double* S, double* E, double* A, double* dS) {
-  return screen_df_sum<L, SLOPE>(F, n, nu, lane, gm, S, E, A, dS);
+__device__ __noinline__ Screened screen_df_sum_call(const float* __restrict__ F, int n, double nu, int lane,
+                                                    unsigned gm) {
+  return screen_df_sum<L, SLOPE>(F, n, nu, lane, gm);
 }
 template <int L>
 __device__ __noinline__ bool stored_sum_slope_call(const double* __restrict__ Ds, const double* __restrict__ us,
@@ -656,18 +668,17 @@ __device__ __forceinline__ bool stored_sum_slope_x(const double* __restrict__ Ds
   if constexpr (NI) return stored_sum_slope_call<L>(Ds, us, n, nu, cf, vf, lane, gm, S, slope);
   else return stored_sum_slope<L>(Ds, us, n, nu, cf, vf, lane, gm, S, slope);
 }
-template <bool NI, int L, bool SLOPE = false>
-__device__ __forceinline__ bool screen_sum_x(const float* __restrict__ Df, const float* __restrict__ uf, int n,
-                                             double nu, int lane, unsigned gm, double* S, double* E, double* A,
-                                             double* dS = nullptr) {
-  if constexpr (NI) return screen_sum_call<L, SLOPE>(Df, uf, n, nu, lane, gm, S, E, A, dS);
-  else return screen_sum<L, SLOPE>(Df, uf, n, nu, lane, gm, S, E, A, dS);
+template <bool NI, int L, bool SLOPE>
+__device__ __forceinline__ Screened screen_sum_x(const float* __restrict__ Df, const float* __restrict__ uf, int n,
+                                                 double nu, int lane, unsigned gm) {
+  if constexpr (NI) return screen_sum_call<L, SLOPE>(Df, uf, n, nu, lane, gm);
+  else return screen_sum<L, SLOPE>(Df, uf, n, nu, lane, gm);
 }
-template <bool NI, int L, bool SLOPE = false>
-__device__ __forceinline__ bool screen_df_sum_x(const float* __restrict__ F, int n, double nu, int lane, unsigned gm,
-                                                double* S, double* E, double* A, double* dS = nullptr) {
-  if constexpr (NI) return screen_df_sum_call<L, SLOPE>(F, n, nu, lane, gm, S, E, A, dS);
-  else return screen_df_sum<L, SLOPE>(F, n, nu, lane, gm, S, E, A, dS);
+template <bool NI, int L, bool SLOPE>
+__device__ __forceinline__ Screened screen_df_sum_x(const float* __restrict__ F, int n, double nu, int lane,
+                                                    unsigned gm) {
+  if constexpr (NI) return screen_df_sum_call<L, SLOPE>(F, n, nu, lane, gm);
+  else return screen_df_sum<L, SLOPE>(F, n, nu, lane, gm);
 }
 
 // The sum and its derivative dS/dnu = sum_j zz_j / t_j^2 = sum_j (u_j / t_j)(Delta_j / t_j) from
@@ -832,6 +843,24 @@ __device__ __forceinline__ double model_root(double t, double F, double psi, dou
   return (dF < 0.0) ? t - F / dF : NAN;
 }
 
+// The next point of the screened probes (any point does; only the number of probes depends on it): the
+// pole model's root, near t by one fixed-point step of dt = F / (1 - dpsi p / (p + dt)), p = t - E,
+// else from its quadratic; F = a0 - t + Psi.
+__device__ __forceinline__ double model_point(double t, double F, double psi, double dpsi, double E, double a0) {
+  const double p = __dsub_rn(t, E);
+  const double d0 = quot_approx(F, __dsub_rn(1.0, dpsi));
+  if (!(p > 0.0) || !(p <= 1.0e300)) return __dadd_rn(t, d0);
+  const double pd = __dadd_rn(p, d0);
+  // |d0| < p / 4 (by the exponents)
+  if (((__double2hiint(d0) & 0x7fffffff) >> 20) + 2 < (__double2hiint(p) >> 20))
+    return __dadd_rn(t, quot_approx(F, __fma_rn(-dpsi, quot_approx(p, pd), 1.0)));
+  const double s = __dmul_rn(__dmul_rn(-dpsi, p), p);
+  const double A = __dsub_rn(__dadd_rn(a0, __fma_rn(dpsi, p, psi)), E);
+  const double disc = root(__fma_rn(A, A, __dmul_rn(4.0, s)));
+  return __dadd_rn(E, is_negative(A) ? quot_approx(__dadd_rn(s, s), __dsub_rn(disc, A))
+                                     : __dmul_rn(0.5, __dadd_rn(A, disc)));
+}
+
 // No screen: every step evaluates phi.
 struct NoScreen {
   __device__ bool operator()(double, double*, double*, int, double* = nullptr, double* = nullptr) const {
@@ -867,8 +896,8 @@ __device__ __forceinline__ bool finish_root(uint64_t lo, uint64_t hi, double sid
     (*steps)++;
     if (!(mag <= finish * t * (a1 + s))) return false;
     const double p = __dsub_rn(t, pole);
-    const double d0 = F / (a1 + s);
-    const double dt = (p < 1e300) ? F / (a1 + s * (p / (p + d0))) : d0;
+    const double d0 = quot_approx(F, a1 + s);
+    const double dt = (p < 1e300) ? quot_approx(F, a1 + s * quot_approx(p, p + d0)) : d0;
     const double tc = __dadd_rn(t, dt);
     if (!(tc >= tlo && tc <= thi)) return false;
     if (dt * dt <= 0x1p-60 * t * p) {
@@ -944,7 +973,10 @@ __device__ double bisect(Phi phi, double side, double floor, double alo, double 
   double Lcl = 0.0, Lch = 0.0;
   // a lower bound on |phi| from a screened value g and its tolerance: |phi - g| <= tol plus
   // roundings of g's size
-  auto lower = [](double g, double tol) { return fmax(fabs(g) * (1.0 - 0x1p-50) - 2.0 * tol, 0.0); };
+  // (zero, a bound too, while the finishing step may still end the solve)
+  auto lower = [&](double g, double tol) {
+    return stop > 1 ? 0.0 : fmax(fabs(g) * (1.0 - 0x1p-50) - 2.0 * tol, 0.0);
+  };
   // an end check: a certified bound, the screen when it settles the point, else phi (*sc: the
   // value is not phi's)
   auto check = [&](uint64_t x, bool* sc, double* lb) -> double {
@@ -1020,7 +1052,7 @@ __device__ double bisect(Phi phi, double side, double floor, double alo, double 
         }
         break;
       }
-      const bool below = below_positive ? (g > 0.0) : (g < 0.0);
+      const bool below = below_positive != is_negative(g);     // a settled g is not zero
       if (below) {
         cl = x;
         Lcl = lower(g, tol);
@@ -1036,11 +1068,14 @@ __device__ double bisect(Phi phi, double side, double floor, double alo, double 
       if (phase == 2) break;
       const double F = below_positive ? g : -g;
       const double slope = dpsi - 1.0;
-      if (!(slope < 0.0)) break;
-      double tc = model_root(t, F, psi, dpsi, pole, a0, 1.0, 1.0);
+      if (!is_negative(slope)) break;
+      double tc = model_point(t, F, psi, dpsi, pole, a0);
       const double tl = dfrom(bl), th = dfrom(bh);
-      if (!(tc > tl && tc < th)) tc = below ? fmin(t + fabs(F / slope), th) : fmax(t - fabs(F / slope), tl);
-      const double dl = 2.0 * tol / -slope;
+      if (dbits(tc) - bl - 1 >= bh - bl - 1) {                  // not inside (also negative or NaN)
+        const double st = fabs(quot_approx(F, slope));
+        tc = below ? fmin(t + st, th) : fmax(t - st, tl);
+      }
+      const double dl = quot_approx(2.0 * tol, -slope);
       if (level == 0 && kScreenDf && fabs(tc - t) <= dl) {
         level = 1;                            // converged at the binary32 screen's resolution
         x = dbits(tc);
@@ -1064,14 +1099,14 @@ __device__ double bisect(Phi phi, double side, double floor, double alo, double 
       if (phase >= cap) { good = false; break; }
       phase++;
       uint64_t mid = lo + ((hi - lo) >> 1);
-      double g, tol, lb = 0.0;
-      bool sc = false;
+      double g = 0.0, tol, lb = 0.0;
+      bool sc = false, below;
       if (mid <= cl || mid >= ch) {
         // a certified bound decides the step
         sc = true;
         ninf++;
-        g = ((mid <= cl) == below_positive) ? 1.0 : -1.0;
-        lb = (mid <= cl) ? Lcl : Lch;
+        below = mid <= cl;
+        lb = below ? Lcl : Lch;
       } else {
         if (scr_on) {
           sc = screen(side * dfrom(mid), &g, &tol, -1, nullptr, nullptr);
@@ -1083,8 +1118,8 @@ __device__ double bisect(Phi phi, double side, double floor, double alo, double 
           nscr++;
           lb = lower(g, tol);
         }
+        below = below_positive ? (g > 0.0) : (g < 0.0);
       }
-      bool below = below_positive ? (g > 0.0) : (g < 0.0);
       if (below) { lo = mid; glo = g; have_lo = true; scr_lo = sc; llo = lb; }
       else { hi = mid; ghi = g; have_hi = true; scr_hi = sc; lhi = lb; }
       it++;
@@ -1265,8 +1300,8 @@ __device__ double accel_solve(Ev ev, double floor, double alo, double ahi, doubl
 // NaN when an argument is not finite (callers then ignore the bound).
 __device__ __forceinline__ double qroot(double B, double E, double W) {
   const double c = E - B;
-  const double s = sqrt(__fma_rn(c, c, 4.0 * W));
-  const double x = (c > 0.0) ? (2.0 * W) / (c + s) : 0.5 * (s - c);
+  const double s = root(__fma_rn(c, c, 4.0 * W));
+  const double x = is_negative(c) ? 0.5 * (s - c) : quot(2.0 * W, c + s);
   return E + x;
 }
 
@@ -1279,8 +1314,8 @@ __device__ __forceinline__ double qroot(double B, double E, double W) {
 __device__ __forceinline__ void quad_bracket(double B, double Efar, double Enear, double W, double* alo,
                                              double* ahi) {
   const double lo = qroot(B, Efar, W), hi = qroot(B, Enear, W);
-  if (isfinite(lo)) *alo = fmax(*alo, lo);
-  if (isfinite(hi)) *ahi = fmin(*ahi, hi);
+  if (finite(lo)) *alo = fmax(*alo, lo);
+  if (finite(hi)) *ahi = fmin(*ahi, hi);
 }
 
 // ---------------------------------------------------------------------------------
@@ -1318,8 +1353,8 @@ struct CornerRule {
 template <int L>
 __device__ __forceinline__ double corner_b(const double* __restrict__ d, const double* __restrict__ zz,
                                            const double* __restrict__ zl, int n, int i,
-                                           double rho, int lane, unsigned gm, double* wn2, CornerRule cr,
-                                           bool* used_dd, double* __restrict__ Ds, double* __restrict__ us,
+                                           double rho, double inv_zi2, int lane, unsigned gm, double* wn2,
+                                           CornerRule cr, bool* used_dd, double* __restrict__ Ds, double* __restrict__ us,
                                            float* __restrict__ F, bool* scr_ok) {
   const double di = d[i];
   bool ok = Ds != nullptr;
@@ -1339,16 +1374,16 @@ __device__ __forceinline__ double corner_b(const double* __restrict__ d, const d
       s2 = __fma_rn(t, r, s2);
     }
     const double P = group_sum<L>(p, gm), N = group_sum<L>(q, gm);
-    *wn2 = group_sum<L>(s2, gm) / zz[i];
-    const double nn = (double)n, sn = sqrt(nn);
-    const double Kb = (1.0 + rho * P - rho * N) / fabs(1.0 + rho * P + rho * N);
-    const double zi = sqrt(zz[i]);
-    const double Kz = (cr.zsum - zi) / zi;
+    *wn2 = group_sum<L>(s2, gm) * inv_zi2;
+    const double nn = (double)n, sn = root(nn);
+    const double rP = rho * P, rN = rho * N;
+    const double Kb = quot((1.0 + rP) - rN, fabs((1.0 + rP) + rN));
+    const double Kz = __fma_rn(cr.zsum, root(inv_zi2), -1.0);
     const double kappa = fmin((nn + 4.0) * sn * Kb, 3.0 * sn + (nn + 4.0) * (1.0 + 2.0 * Kz));
     *scr_ok = !group_any<L>(!ok, gm);
     if (kappa <= cr.T_kappa * nn) {
       *used_dd = false;
-      return (1.0 / zz[i]) * ((1.0 / rho + P) + N);
+      return inv_zi2 * ((1.0 / rho + P) + N);
     }
   }
   *used_dd = true;
@@ -1388,14 +1423,14 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
   bool used_dd, rng_ok = false;
   // the binary32 copies and low parts follow the two binary64 arrays (us = Ds + n)
   float* const F = (Ds && screen && !fast) ? (float*)(us + n) : nullptr;
-  double b = corner_b<L>(d, zz, zl, n, i, rho, lane, gm, &wn2, cr, &used_dd, Ds, us, F, &rng_ok);
+  const double inv_zi2 = 1.0 / zz[i];
+  double b = corner_b<L>(d, zz, zl, n, i, rho, inv_zi2, lane, gm, &wn2, cr, &used_dd, Ds, us, F, &rng_ok);
   const bool scr_ok = rng_ok && F;
   double side = (i == k) ? 1.0 : -1.0;
   double di = d[i];
-  double inv_zi2 = 1.0 / zz[i];
   // Weyl: the extreme eigenvalue lies within ||w|| of max(b, max delta) (rightmost) or
   // min(b, min delta) (leftmost); Rayleigh: nu >= b (rightmost), nu <= b (leftmost).
-  double wn = sqrt(wn2);
+  double wn = root(wn2);
   // floor: the pole of g next to the extreme eigenvalue (largest delta_j for the
   // rightmost, smallest for the leftmost), or 0 when all poles lie on the other side.
   double floor, E;   // E: the nearest pole on |nu| (the accelerated solve's model pole)
@@ -1409,25 +1444,25 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
   // pole b ~ 1/zeta_i^2 dominates and this bracket is narrow.
   if (side > 0) {
     // largest delta_j: the nearest pole above d_i, or for i = 0 the farthest pole below
-    double dmax = (i > 0) ? 1.0 / (d[i - 1] - di) : (n > 1 ? 1.0 / (d[n - 1] - di) : -INFINITY);
+    double dmax = (i > 0) ? quot(1.0, d[i - 1] - di) : (n > 1 ? quot(1.0, d[n - 1] - di) : -INFINITY);
     floor = fmax(dmax, 0.0);
     E = dmax;
     rlo = b;
     rhi = fmax(b, dmax) + wn;
-    if (b > dmax) rhi = fmin(rhi, b + wn2 / (b - dmax));
+    if (b > dmax) rhi = fmin(rhi, b + quot(wn2, b - dmax));
     // smallest delta_j: the nearest pole below d_i, or for i = n-1 the farthest pole above
-    const double dmin = (i + 1 < n) ? 1.0 / (d[i + 1] - di) : (n > 1 ? 1.0 / (d[0] - di) : -INFINITY);
+    const double dmin = (i + 1 < n) ? quot(1.0, d[i + 1] - di) : (n > 1 ? quot(1.0, d[0] - di) : -INFINITY);
     quad_bracket(b, dmin, dmax, wn2, &rlo, &rhi);
   } else {
-    double dmin = (i + 1 < n) ? 1.0 / (d[i + 1] - di) : INFINITY;
+    double dmin = (i + 1 < n) ? quot(1.0, d[i + 1] - di) : INFINITY;
     floor = fmax(-dmin, 0.0);
     // smallest delta_j: the nearest pole below d_i, or for i = n-1 the farthest pole above
-    E = (i + 1 < n) ? -dmin : (n > 1 ? -1.0 / (d[0] - di) : -INFINITY);
+    E = (i + 1 < n) ? -dmin : (n > 1 ? quot(-1.0, d[0] - di) : -INFINITY);
     rlo = -b;
     rhi = -fmin(b, dmin) + wn;
-    if (b < dmin) rhi = fmin(rhi, -b + wn2 / (dmin - b));
+    if (b < dmin) rhi = fmin(rhi, -b + quot(wn2, dmin - b));
     // on t = -nu the poles are -delta_j: the nearest is -dmin, the farthest -(largest delta_j)
-    const double dmx = (i > 0) ? 1.0 / (d[i - 1] - di) : (n > 1 ? 1.0 / (d[n - 1] - di) : INFINITY);
+    const double dmx = (i > 0) ? quot(1.0, d[i - 1] - di) : (n > 1 ? quot(1.0, d[n - 1] - di) : INFINITY);
     quad_bracket(-b, -dmx, -dmin, wn2, &rlo, &rhi);
   }
   alo = fmax(alo_in, rlo);
@@ -1480,16 +1515,14 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
       return __dsub_rn(__dsub_rn(b, v), __dmul_rn(S, inv_zi2));
     };
     // The screen settles a step when its g = fl(fl(b - v) - fl(Sx inv_zi2)) exceeds every
-    // way the decision could differ from phi's: |Sx - S| <= Ex (the screen's bound),
-    // |S64 - S| <= stored_sum_error for phi's binary64 sum, and the roundings of the two
-    // products.  fl(x - y) has the sign of x - y, so phi's sign then equals the sign of g.
-    const double mlane = (double)((n + L - 1) / L);
-    auto decide = [&](double Sx, double Ex, double aS, double v, double* g, double* tl) -> bool {
-      const double E64 = stored_sum_error<L>(mlane, aS);
-      const double tol = 1.01 * inv_zi2 * (Ex + E64 + 0x1p-51 * aS);
-      const double G = __dsub_rn(__dsub_rn(b, v), __dmul_rn(Sx, inv_zi2));
-      if (!(fabs(G) > tol)) return false;
-      if (fabs(G) <= 2.0 * tol) r.screened_near++;
+    // way the decision could differ from phi's: the screen's bound x on |Sx - S64| for phi's
+    // binary64 sum, with the roundings of the two products.  fl(x - y) has the sign of x - y, so
+    // phi's sign then equals the sign of g.
+    auto decide = [&](const Screened& c, double v, double Sz, double* g, double* tl) -> bool {
+      const double tol = __dmul_rn(inv_zi2, (double)c.x);
+      const double G = __dsub_rn(__dsub_rn(b, v), Sz);
+      if (!mag_greater(G, tol)) return false;
+      if (!mag_greater(G, __dadd_rn(tol, tol))) r.screened_near++;
       *g = G;
       *tl = tol;
       return true;
@@ -1499,12 +1532,13 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
     int f32_fail = 0;
     auto scr = [&](double v, double* g, double* tl, int mode, double* psi, double* dpsi) -> bool {
       if (!scr_ok) return false;
-      double Sx, Ex, aS, dS = 0.0;
+      Screened c;
+      double Sz = 0.0;
       bool ok = false;
       if (mode == 0 || (mode < 0 && f32_fail < kScreen32Tries)) {
-        ok = (psi ? screen_sum_x<NI, L, true>(F, F + n, n, v, lane, gm, &Sx, &Ex, &aS, &dS)
-                  : screen_sum_x<NI, L>(F, F + n, n, v, lane, gm, &Sx, &Ex, &aS)) &&
-             decide(Sx, Ex, aS, v, g, tl);
+        c = psi ? screen_sum_x<NI, L, true>(F, F + n, n, v, lane, gm) : screen_sum_x<NI, L, false>(F, F + n, n, v, lane, gm);
+        Sz = __dmul_rn(c.S, inv_zi2);
+        ok = decide(c, v, Sz, g, tl);
         if (ok) {
           if (mode < 0) f32_fail = 0;
         } else {
@@ -1514,17 +1548,16 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
       }
       if (!ok) {
         if (mode == 1) f32_fail = kScreen32Tries;   // the probes have reached the binary32 window
-        ok = kScreenDf &&
-             (psi ? screen_df_sum_x<NI, L, true>(F, n, v, lane, gm, &Sx, &Ex, &aS, &dS)
-                  : screen_df_sum_x<NI, L>(F, n, v, lane, gm, &Sx, &Ex, &aS)) &&
-             decide(Sx, Ex, aS, v, g, tl);
-        if (!ok) return false;
+        if (!kScreenDf) return false;
+        c = psi ? screen_df_sum_x<NI, L, true>(F, n, v, lane, gm) : screen_df_sum_x<NI, L, false>(F, n, v, lane, gm);
+        Sz = __dmul_rn(c.S, inv_zi2);
+        if (!decide(c, v, Sz, g, tl)) return false;
         r.screened_df++;
       }
       // Psi and Psi' on t = |nu| as the accelerated solve forms them (F = side b - t + Psi)
       if (psi) {
-        *psi = -side * __dmul_rn(Sx, inv_zi2);
-        *dpsi = -__dmul_rn(dS, inv_zi2);
+        *psi = -side * Sz;
+        *dpsi = -__dmul_rn((double)c.slope, inv_zi2);
       }
       return true;
     };
