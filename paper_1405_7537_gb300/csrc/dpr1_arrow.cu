@@ -943,7 +943,16 @@ static size_t arrow_term_bytes(int64_t n) {
 template <int L>
 static dpr1_status launch_arrow(int n, const double* d, const double* z, ArrowWs* w, const Options& o, char* tail,
                                 size_t tb, double* Vt, int64_t ldv, cudaStream_t st) {
-  const int groups_per_block = (32 * o.warps) / L;
+  // fewer lane groups than 8-warp blocks on every SM hold: blocks of fewer warps, one per SM
+  int warps = o.warps;
+  if (o.warps_auto && o.bps_auto) {
+    const int64_t w_need = (((int64_t)n + 1) * L + 32 * (int64_t)sm_count() - 1) / (32 * (int64_t)sm_count());
+    // no more lane groups (a last block rounds up) than the default launch's, which have buffers
+    const int64_t most = ((int64_t)n + 1 + 256 / L - 1) / (256 / L) * (256 / L);
+    warps = w_need < 8 ? (int)w_need : 8;
+    while (warps < 8 && ((int64_t)n + 32 * warps / L) / (32 * warps / L) * (32 * warps / L) > most) warps++;
+  }
+  const int groups_per_block = (32 * warps) / L;
   int64_t want = ((int64_t)n + 1 + groups_per_block - 1) / groups_per_block;
   int grid = sm_count() * o.bps;
   if (want < grid) grid = (int)(want > 0 ? want : 1);
@@ -952,7 +961,7 @@ static dpr1_status launch_arrow(int n, const double* d, const double* z, ArrowWs
     // formed the same way whichever group takes an eigenvalue)
     const int64_t tn = ((int64_t)n + 31) & ~(int64_t)31;
     const int64_t slots = (int64_t)(tb / (TERM_BYTES * (size_t)tn));
-    const int64_t need = arrow_groups(n, L, o.warps, o.bps);
+    const int64_t need = arrow_groups(n, L, warps, o.bps);
     if (slots >= need) {
       w->terms = (double*)tail;
       w->term_n = tn;
@@ -970,7 +979,7 @@ static dpr1_status launch_arrow(int n, const double* d, const double* z, ArrowWs
       }
     }
   }
-  k_arrow_solve<L><<<grid, 32 * o.warps, 0, st>>>(n, d, z, *w, o.cap, o.fast, o.screen, Vt, ldv);
+  k_arrow_solve<L><<<grid, 32 * warps, 0, st>>>(n, d, z, *w, o.cap, o.fast, o.screen, Vt, ldv);
   return DPR1_OK;
 }
 

@@ -1290,12 +1290,13 @@ static dpr1_status run_table(const Prob& pb, void* workspace, size_t wbytes, con
   if (dg > sms * 8) dg = sms * 8;
   k_deflate<<<dg > 0 ? dg : 1, 128, 0, st>>>(pb, w);
   int L = o.lanes ? o.lanes : default_lanes(avg_n, pb.P);
-  // Shape of the solve kernel.  Its time is set by the binary64 pipe of the busiest SM, so the
-  // eigenvalues must spread evenly over the SMs: with fewer lane groups than 8-warp blocks on
-  // every SM can hold, blocks of fewer warps, at most one per SM; else as many 8-warp blocks per
-  // SM (up to the default, all resident at once) as the lane groups fill completely, whose
-  // groups take eigenvalues from the work counter (a partly filled extra block per SM would load
-  // some SMs more than others).  Options may fix the shape.
+  // Shape of the solve kernel.  Its time is set by the latency of an eigenvalue's passes and the
+  // binary64 pipe of the busiest SM, so the eigenvalues must spread evenly over the SMs.  Where every
+  // lane group can be resident at once (w_need warps per SM, up to 8 for each block of the form), one
+  // wave of equal blocks holds them all: as few blocks per SM as 8 warps each allow, of as many warps
+  // as that takes.  (With the 8-warp blocks that the lane groups fill completely, the eigenvalues left
+  // over ran as a second wave at twice the latency.)  Beyond that, 8-warp blocks, all resident at once,
+  // whose groups take eigenvalues from the work counter.  Options may fix the shape.
   int warps = o.warps;
   int bps = o.bps;
   // problems of small order run the solve kernel compiled for fewer resident blocks (its sums
@@ -1305,10 +1306,15 @@ static dpr1_status run_table(const Prob& pb, void* workspace, size_t wbytes, con
   const int64_t lanes_total = pb.total * L;
   if (o.warps_auto) {
     const int64_t w_need = (lanes_total + 32 * (int64_t)sms - 1) / (32 * (int64_t)sms);
-    warps = w_need >= 8 ? 8 : (int)(w_need > 0 ? w_need : 1);
-    if (o.bps_auto) {
-      const int64_t fill = lanes_total / ((int64_t)32 * 8 * sms);
-      if (fill < bps) bps = fill > 1 ? (int)fill : 1;
+    if (w_need <= 8) {
+      warps = (int)(w_need > 0 ? w_need : 1);
+      if (o.bps_auto) bps = 1;
+    } else {
+      warps = 8;
+      if (o.bps_auto && w_need <= 8 * bps) {
+        bps = (int)((w_need + 7) / 8);
+        warps = (int)((w_need + bps - 1) / bps);
+      }
     }
   }
   int groups_per_block = (32 * warps) / L;
