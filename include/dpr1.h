@@ -195,7 +195,9 @@ DPR1_API dpr1_status dpr1_eig_batched(int64_t nprob, int64_t total_n, const int6
 /*
  * Bytes of workspace for dpr1_eig_backward on order n (256-byte aligned, uninitialised):
  * three rows of n doubles (partial rows of the gradients of d and z, and the current row's
- * reciprocals) for each of 1064, 2128 or 3192 warps (n <= 8192, <= 24576, above).
+ * reciprocals) for each of 1064, 2128, 2432 or 3648 warps (n <= 3072, <= 10240, <= 24576, above).
+ * A workspace for 1064, 2128 or 3192 warps (n <= 8192, <= 24576, above) is accepted too; the sums then
+ * have fewer partial rows, so results may differ in their last bits.
  */
 DPR1_API size_t dpr1_backward_workspace_size(int64_t n);
 
