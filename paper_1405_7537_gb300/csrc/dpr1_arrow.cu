@@ -908,7 +908,8 @@ __global__ void k_arrow_one(double alpha, double* lambda, double* Vt, double* si
 }
 
 // lane groups of the solve kernel's default launch and of the remedies kernel
-static int arrow_lanes(int64_t n) { return n <= 96 ? 8 : (n <= 384 ? 16 : 32); }
+// (a warp per eigenvalue, as for one problem D + rho z z^T)
+static int arrow_lanes(int64_t) { return 32; }
 
 static int64_t arrow_groups(int64_t n, int L, int warps, int bps) {
   const int groups_per_block = (32 * warps) / L;

@@ -56,9 +56,10 @@
 #define DPR1_FIX_WARP_MAX_N 2048
 #endif
 // and so do fewer problems up to this mean size (each flagged eigenvalue's evaluations are then
-// short, and a block-wide group would pay a barrier per evaluation)
+// short, and a block-wide group would pay a barrier per evaluation: n = 512, 800, 1024 take 124, 167
+// and 195 us with warps, 138, 191 and 134 with blocks)
 #ifndef DPR1_FIX_SMALL_N
-#define DPR1_FIX_SMALL_N 1024
+#define DPR1_FIX_SMALL_N 900
 #endif
 // eigenvector rows as pairs of components with 16-byte accesses
 #ifndef DPR1_VEC_PAIRS
@@ -142,14 +143,14 @@ size_t ws_layout2(int64_t total, int64_t nprob, bool batched, Ws* w, char* base)
   return off;
 }
 
-// Lane-group width of k_solve for an average problem order (when the options leave it open).  In a
+// Lane-group width of k_solve for an average problem order (when the options leave it open).  One
+// problem always takes a warp per eigenvalue: small ones leave most of the GPU idle, and the time is
+// the latency of an eigenvalue's passes and the divergence of the groups that share a warp (n = 16, 96,
+// 384: 92, 123 and 274 us for the kernel with 8, 8 and 16 lanes, 55, 66 and 183 with 32).  In a
 // batch, eight lanes up to a mean order of 384 (problems of orders 96-384: 33.3 ms against 39.8 with
 // 16 lanes and 48.3 with 32 for 425k eigenpairs; orders 16-96: 18.2 against 24.9 and 32.5) and a
 // warp above (orders 384-2048: 108.4 ms against 115.8 with 16 lanes and 140.3 with 8).
-static int default_lanes(double avg_n, int64_t nprob = 1) {
-  if (nprob > 1) return avg_n <= 384 ? 8 : 32;
-  return avg_n <= 96 ? 8 : (avg_n <= 384 ? 16 : 32);
-}
+static int default_lanes(double avg_n, int64_t nprob = 1) { return nprob > 1 && avg_n <= 384 ? 8 : 32; }
 
 // Bytes of the stored-element buffers appended to the workspace: TERM_BYTES term_n bytes for
 // each lane group of k_solve's default launch (8 warps per block, DPR1_SOLVE_MIN_BLOCKS blocks per
