@@ -5,11 +5,11 @@
 //   (Sec. 2.3): the corner b of Eq. (b_ob), and f(sigma) / the denominator of gamma
 //   for the non-pole shifts (R2, Eq. (gamma)).  Error-free transformations: Knuth's
 //   TwoSum, Dekker's FastTwoSum and the exact product through fma.
-// * a binary64 reciprocal: the sm_103a approximate reciprocal instruction
-//   (rcp.approx.ftz.f64, about 20 correct bits) refined by one third-order
-//   Newton-Raphson step r = r0 (1 + e + e^2), e = 1 - x r0; the result is within
-//   one unit in the last place of 1/x for |x| in [2^-1020, 2^1020] (outside that
-//   range the IEEE quotient is used).
+// * a binary64 reciprocal within one unit in the last place of 1/x for |x| in
+//   [2^-1020, 2^1020] (outside that range the IEEE quotient is used): a Newton step on a
+//   seed from binary32 and integer arithmetic (the loops over the terms), or one
+//   third-order step r = r0 (1 + e + e^2), e = 1 - x r0, on the sm_103a approximate
+//   reciprocal instruction (rcp.approx.ftz.f64, about 20 correct bits).
 // * lane-group reductions with xor shuffles: every lane of a group ends with the
 //   bit-identical total (IEEE addition is commutative), so every lane takes the
 //   same bisection decisions without a broadcast.
@@ -83,12 +83,35 @@ __device__ __forceinline__ float rcp_approx_f32(float x) {
   return r;
 }
 
-// 1/x within one ulp for |x| in [2^-1020, 2^1021) (see the file comment); no range handling.
-__device__ __forceinline__ double rcp_nr(double x) {
+// 1/x within one ulp for |x| in [2^-1020, 2^1021) (see the file comment); no range handling.  The
+// shortest chain, for the scalar work.
+__device__ __forceinline__ double rcp_chain(double x) {
   double r0 = rcp_approx(x);
   double e = __fma_rn(-x, r0, 1.0);
   double p = __fma_rn(e, e, e);
   return __fma_rn(r0, p, r0);
+}
+
+// The same for the loops over the terms, with one binary64 instruction less: a seed within 2^-45 formed
+// on the other pipes, where an instruction costs a 64th, leaves one Newton step.  With x's mantissa
+// m = mh + ml in [1, 2) (mh its leading 24 bits), r0 = 1/mh in (1/2, 1] from the binary32
+// approximation and t = 1 - m r0 in binary32 (|t| < 2^-22, within 2^-47), r0 + r0 t is 1/m within
+// t^2 + 2^-47; r0 t is added to the bits of r0 as a binary64 number in units of 2^-53 (for r0 = 1,
+// t <= 0, and the units below 1 are 2^-53 too), and the exponent and sign of x are applied to the bits.
+// The Newton step squares the error, so the result is within 0.51 ulp.
+__device__ __forceinline__ double rcp_nr(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const float mh = __uint_as_float((__funnelshift_l(lo, hi, 3) & 0x7fffffu) | 0x3f800000u);
+  const float ml = __fmul_rn(__int2float_rn((int)(lo & 0x1fffffffu)), 0x1p-52f);
+  const float r0 = rcp_approx_f32(mh);
+  const float t = __fmaf_rn(-ml, r0, __fmaf_rn(-mh, r0, 1.0f));
+  const int k = __float2int_rn(__fmul_rn(__fmul_rn(r0, t), 0x1p53f));
+  const unsigned rb = __float_as_uint(r0);
+  const long long m = (((long long)(rb >> 3) + 0x38000000ll) << 32) + (long long)((unsigned long long)(rb << 29)) + k;
+  const unsigned ex = (hi & 0x7ff00000u) - 0x3ff00000u;
+  const double r = __hiloint2double((int)(((unsigned)(m >> 32) - ex) ^ (hi & 0x80000000u)), (int)m);
+  const double e = __fma_rn(-x, r, 1.0);
+  return __fma_rn(r, e, r);
 }
 
 // the exponent field of x lies in [1023-1020, 1023+1020]: rcp_nr is within one ulp
@@ -117,7 +140,9 @@ __device__ __forceinline__ double rcp(double x) { return rcp_in_range(x) ? rcp_n
 // rcp_nr's range); quot_approx: within 2^-38 (the seed's 2^-20 and one Newton step), NaN or infinity out
 // of range, which its callers treat as "no point".  root: sqrt(x) within 2 ulps by two Newton steps on the
 // hardware's reciprocal square root, sqrt out of line for the rest.
-__device__ __forceinline__ double quot(double a, double b) { return __dmul_rn(a, rcp(b)); }
+__device__ __forceinline__ double quot(double a, double b) {
+  return __dmul_rn(a, rcp_in_range(b) ? rcp_chain(b) : rcp_ieee(b));
+}
 __device__ __forceinline__ double quot_approx(double a, double b) {
   const double r = rcp_approx(b);
   return __dmul_rn(a, __fma_rn(r, __fma_rn(-b, r, 1.0), r));
