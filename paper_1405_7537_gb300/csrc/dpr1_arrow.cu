@@ -55,6 +55,8 @@ struct ArrowWs {
   int* shift;                    // pole index, -1 for a non-pole shift
   int* list;                     // eigenvalues flagged by K_nu
   double* fixinfo;               // per flagged slot: K_nu, K_nu at the other pole, distance ratio
+  long long* dq;                 // for the shift tests, in fixinfo's bytes before it is filled (as Ws::dq)
+  float* zf;
   int* zlist;                    // near-zero candidates
   double* lamz;                  // lambda recomputed from A^{-1} (NaN: not recomputed)
   double* ds;                    // d' = 2^-a d and z' = 2^-a z (normalised copies)
@@ -97,6 +99,8 @@ static size_t arrow_layout(int64_t n, ArrowWs* w, char* base) {
     w->shift = (int*)(base + o_sh);
     w->list = (int*)(base + o_l);
     w->fixinfo = (double*)(base + o_fi);
+    w->dq = (long long*)(base + o_fi);
+    w->zf = (float*)(base + o_fi + 8 * nn);
     w->zlist = (int*)(base + o_zl2);
     w->lamz = (double*)(base + o_lz);
     w->ds = (double*)(base + o_ds);
@@ -159,6 +163,8 @@ __global__ void k_arrow_check(int n, const double* __restrict__ d, const double*
     const double zq = __dmul_rn(zj, zj);
     zz[j] = zq;
     zl[j] = __fma_rn(zj, zj, -zq);
+    w.dq[j] = pole_int(w.ds[j]);
+    w.zf[j] = weight_f32(zq);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0 && !isfinite(alpha)) bits |= ST_NONFINITE;
   bits = __reduce_or_sync(FULL, bits);
@@ -471,7 +477,7 @@ __global__ void __launch_bounds__(256, DPR1_SOLVE_MIN_BLOCKS) k_arrow_solve(int 
       const double tau = __dmul_rn(__dsub_rn(d[k - 1], dk), 0.5);
       const double c = __dsub_rn(__dsub_rn(alpha, dk), tau);
       double sp = 0.0, sn = 0.0, F = 0.0;
-      const int sf = (kArrowShift32 && screen) ? shift_test_arrow_f32<L>(d, zz, n, dk, tau, c, lane, gm) : 0;
+      const int sf = (kArrowShift32 && screen) ? shift_test_arrow_f32<L>(w.dq, w.zf, n, k, tau, c, lane, gm) : 0;
       shift32 = sf != 0;
       if (!shift32) {
         for (int j = lane; j < n; j += L) {

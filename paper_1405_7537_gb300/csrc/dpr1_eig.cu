@@ -131,6 +131,8 @@ size_t ws_layout2(int64_t total, int64_t nprob, bool batched, Ws* w, char* base)
     w->gst = (int*)gst; w->rprev = (double*)rprev; w->rcur = (double*)rcur; w->dlist = (int*)dlist;
     w->zlist = (int*)zlist;
     w->fixinfo = (double*)fk;
+    w->dq = (long long*)fk;
+    w->zf = (float*)(fk + sizeof(double) * nn);
     w->pexp = (int*)pe;
     w->prho = (double*)pr;
     w->pzsum = (double*)pzs;
@@ -320,6 +322,8 @@ __global__ void k_scan(Prob pb, Ws w) {
     const double zq = __dmul_rn(zjs, zjs);
     w.zz[g] = zq;
     w.zl[g] = __fma_rn(zjs, zjs, -zq);
+    w.dq[g] = pole_int(djs);
+    w.zf[g] = weight_f32(zq);
   }
   bits = __reduce_or_sync(FULL, bits);
   if ((threadIdx.x & 31) == 0 && bits) atomicOr(w.status, bits);
@@ -369,6 +373,8 @@ __device__ int deflate_group(const Ws& w, int64_t base, const double* d, const d
     const double zq = __dmul_rn(zs, zs);
     w.zz[base + *nr] = zq;
     w.zl[base + *nr] = __fma_rn(zs, zs, -zq);
+    w.dq[base + *nr] = pole_int(w.dr[base + *nr]);
+    w.zf[base + *nr] = weight_f32(zq);
     (*nr)++;
   }
   return e + 1;
@@ -419,6 +425,8 @@ __global__ void k_deflate(Prob pb, Ws w) {
             const double zz = __dmul_rn(zq, zq);
             w.zz[base + r] = zz;
             w.zl[base + r] = __fma_rn(zq, zq, -zz);
+            w.dq[base + r] = pole_int(scalbn(dq, -ea));
+            w.zf[base + r] = weight_f32(zz);
           }
         }
         nr += __popc(km);
@@ -642,7 +650,7 @@ __global__ void __launch_bounds__(256, MINB)
       double tau = __dmul_rn(__dsub_rn(d[k - 1], dk), 0.5);
       double sp = 0.0, sn = 0.0, F = 0.0;
       // the binary32 pass decides where its bound settles the sign (the binary64 pass's sign)
-      const int sf = (kShift32 && screen) ? shift_test_f32<L>(d, zz, n, dk, tau, rho, lane, gm) : 0;
+      const int sf = (kShift32 && screen) ? shift_test_f32<L>(w.dq + base, w.zf + base, n, k, tau, rho, lane, gm) : 0;
       shift32 = sf != 0;
       if (sf == 0) {
         for (int j = lane; j < n; j += L) {

@@ -48,6 +48,10 @@ struct Ws {
   int* dlist;                 // deflated positions, increasing
   int* zlist;                 // near-zero candidates
   double* fixinfo;            // per flagged slot: K_nu, K_nu at the other pole, distance ratio
+  // the reduced problem for the shift tests of the solve kernel (in fixinfo's bytes, which the
+  // classification fills after it): d in units of 2^-62 and z^2 in binary32
+  long long* dq;
+  float* zf;
   int* pexp;                  // [2P]: exponents (a, b) of the normalisation D' = 2^-a D, z' = 2^-b z
   double* prho;               // [P]: rho' = 2^(2b - a) rho
   double* pzsum;              // [P]: sum_j |zeta'_j| (for K_z of Eq. (knu2))

@@ -375,40 +375,44 @@ __device__ __forceinline__ float rn32(double x, bool* ok) {
   return *ok ? __uint_as_float(sgn | ((unsigned)ef << 23) | (q & 0x7fffffu)) : 0.0f;
 }
 
-// Shift test of Algorithm 1 in binary32: F = 1 + rho sum_j zz_j / ((d_j - d_k) - tau).  Each lane
-// forms Delta_j = fl(d_j - d_k) in binary64 (one subtraction) and the rest in binary32 from
-// Df = RN32(Delta_j), zf = RN32(zz_j), tf = RN32(tau) (integer conversions): den = fl(Df - tf),
-// r = 1/den (approximate reciprocal and one Newton step, 1.07 eps), t = fl(zf r), summed by Sum2.
-// With eps = 2^-24, |den - ((d_j - d_k) - tau)| <= eps (|Df| + tf) (1 + 2^-28) + eps |den| and
-// w = (|Df| + tf) |r|, the term is within e_j = |t| eps (1.01 w + 4.2) of zz_j / ((d_j - d_k) - tau)
-// (the conversions of zz and Delta, the reciprocal, the product and Sum2's share), valid while
-// w <= 2^20 (else the lane reports failure); a weight below the binary32 range (zf = 0) adds at
-// most 2^-125 |r|.  shift_sum_f32 returns the sum S32 with es = sum e_j and as = sum |t_j| (each
-// rounded up); the tests below bound |F32 - F| for the exact F and |F64 - F| for the binary64 pass
+// Shift test of Algorithm 1 in binary32: F = 1 + rho sum_j zz_j / ((d_j - d_k) - tau), from
+// q_j = d_j in units of 2^-62 (the poles are normalised, |d_j| < 1; rounded to an integer) and
+// zf_j = RN32(zz_j), both stored once per problem: no binary64 operation per term.  With eps = 2^-24 each
+// lane forms Df = RN32(q_j - q_k), within eps |Df| and one unit of d_j - d_k, and tf = RN32(tau), both in
+// units of 2^-62, and den = fl(Df - tf), r = 1/den (approximate reciprocal and one Newton step, 1.07
+// eps), t = fl(zf r), summed by Sum2.  |den - ((d_j - d_k) - tau)| <= eps (|Df| + tf) (1 + 2^-23) + eps |den|
+// + 1, so with w = (|Df| + tf) |r| the term is within e_j = |t| eps (1.01 w + 4.2 + 1.01 |r| / eps) of
+// zz_j / ((d_j - d_k) - tau) (the conversion of zz, the reciprocal, the product and Sum2's share
+// included), valid while w <= 2^19 and |r| <= 2^-6 (else the lane reports failure; poles closer than
+// about 2^-40 leave the sign to the binary64 pass more often); a weight below the binary32 range
+// (zf = 0) adds at most 2^-125 |r|.  shift_sum_f32 returns the sum S32 with es = sum e_j / eps and as = sum
+// |t_j|; the tests below bound |F32 - F| for the exact F and |F64 - F| for the binary64 pass
 // of the solve kernel (two roundings of each difference, the one-ulp reciprocal and the product:
 // u (w + 4) per term, m = ceil(n / L) accumulations per lane, the tree and the last sum), so a
 // decision on the sign of F32 with |F32| > E is the binary64 pass's decision.
 template <int L>
-__device__ __forceinline__ bool shift_sum_f32(const double* __restrict__ d, const double* __restrict__ zz, int n,
-                                              double dk, double tau, int lane, unsigned gm, double* S, float* es_out,
+__device__ __forceinline__ bool shift_sum_f32(const long long* __restrict__ q, const float* __restrict__ zf, int n,
+                                              int k, double tau, int lane, unsigned gm, double* S, float* es_out,
                                               float* as_out) {
   bool ok = true;
-  const float tf = rn32(tau, &ok);
+  const float tf = rn32(__dmul_rn(tau, 0x1p62), &ok);
+  const long long qk = q[k];
   float sh = 0.0f, sl = 0.0f, e = 0.0f, a1 = 0.0f;
   for (int j = lane; j < n; j += L) {
-    bool okd, okz;
-    const float Df = rn32(__dsub_rn(d[j], dk), &okd);
-    const float zf = rn32(zz[j], &okz);
+    const float Df = __ll2float_rn(q[j] - qk);
+    const float z = zf[j];
     const float den = __fsub_rn(Df, tf);
     const float r0 = rcp_approx_f32(den);
     const float r = __fmaf_rn(r0, __fmaf_rn(-den, r0, 1.0f), r0);
-    const float t = __fmul_rn(zf, r);
+    // the weight in units of 2^-62 too, as two exact powers around the reciprocal
+    const float rs = __fmul_rn(r, 0x1p62f);
+    const float t = __fmul_rn(z, rs);
     const float ar = fabsf(r);
     const float w = __fmul_rn(__fadd_rn(fabsf(Df), tf), ar);
-    ok &= okd && (w <= 0x1p20f);
+    ok &= (w <= 0x1p19f) && (ar <= 0x1p-6f);
     const float at = fabsf(t);
-    e = __fmaf_rn(at, __fmaf_rn(1.01f, w, 4.2f), e);
-    if (!okz) e = __fmaf_rn(ar, 0x1p-125f, e);
+    e = __fmaf_rn(at, __fmaf_rn(1.01f, w, __fmaf_rn(1.01f * 0x1p24f, ar, 4.2f)), e);
+    if (z == 0.0f) e = __fmaf_rn(fabsf(rs), 0x1p-101f, e);
     a1 = __fadd_rn(a1, at);
     float er;
     sh = two_sum_f(sh, t, &er);
@@ -420,6 +424,13 @@ __device__ __forceinline__ bool shift_sum_f32(const double* __restrict__ d, cons
   *es_out = group_sum_f<L>(e, gm);
   *as_out = group_sum_f<L>(a1, gm);
   return !group_any<L>(!ok, gm);
+}
+
+// the stored forms of a normalised pole and of a weight's square
+__device__ __forceinline__ long long pole_int(double d) { return __double2ll_rn(__dmul_rn(d, 0x1p62)); }
+__device__ __forceinline__ float weight_f32(double zz) {
+  bool ok;
+  return rn32(zz, &ok);
 }
 
 // The bound of |S32 - S| and |S64 - S| together, rounded up (the factor 1 + 2^-18 covers the roundings
@@ -437,11 +448,11 @@ __device__ __forceinline__ float shift_bound(int n, float es, float as) {
 
 // D + rho z z^T: the sign (+1, -1) of F = 1 + rho S, 0 where the bound leaves it open.
 template <int L>
-__device__ __noinline__ int shift_test_f32(const double* __restrict__ d, const double* __restrict__ zz, int n,
-                                           double dk, double tau, double rho, int lane, unsigned gm) {
+__device__ __noinline__ int shift_test_f32(const long long* __restrict__ q, const float* __restrict__ zf, int n,
+                                           int k, double tau, double rho, int lane, unsigned gm) {
   double S;
   float es, as;
-  const bool ok = shift_sum_f32<L>(d, zz, n, dk, tau, lane, gm, &S, &es, &as);
+  const bool ok = shift_sum_f32<L>(q, zf, n, k, tau, lane, gm, &S, &es, &as);
   const double F = __fma_rn(rho, S, 1.0);
   const double E = __fma_rn(rho, (double)shift_bound<L>(n, es, as), 0x1p-49);
   return (ok && es < INFINITY && mag_greater(F, E)) ? (is_negative(F) ? -1 : 1) : 0;
@@ -451,11 +462,11 @@ __device__ __noinline__ int shift_test_f32(const double* __restrict__ d, const d
 // binary64 pass subtracts its sum fl(sp + sn) from; fl(c - x) has the sign of c - x, so the
 // binary64 decision is the sign of c - fl(sp + sn), within the same bound of c - S32.
 template <int L>
-__device__ __noinline__ int shift_test_arrow_f32(const double* __restrict__ d, const double* __restrict__ zz, int n,
-                                                 double dk, double tau, double c, int lane, unsigned gm) {
+__device__ __noinline__ int shift_test_arrow_f32(const long long* __restrict__ q, const float* __restrict__ zf,
+                                                 int n, int k, double tau, double c, int lane, unsigned gm) {
   double S;
   float es, as;
-  const bool ok = shift_sum_f32<L>(d, zz, n, dk, tau, lane, gm, &S, &es, &as);
+  const bool ok = shift_sum_f32<L>(q, zf, n, k, tau, lane, gm, &S, &es, &as);
   const double F = __dsub_rn(c, S);
   const double E = __fma_rn(0x1p-49, fabs(c), (double)shift_bound<L>(n, es, as));
   return (ok && es < INFINITY && mag_greater(F, E)) ? (is_negative(F) ? -1 : 1) : 0;
