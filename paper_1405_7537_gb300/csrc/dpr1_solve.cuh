@@ -854,22 +854,34 @@ __device__ __forceinline__ double model_root(double t, double F, double psi, dou
   return (dF < 0.0) ? t - F / dF : NAN;
 }
 
-// The next point of the screened probes (any point does; only the number of probes depends on it): the
-// pole model's root, near t by one fixed-point step of dt = F / (1 - dpsi p / (p + dt)), p = t - E,
-// else from its quadratic; F = a0 - t + Psi.
+// x / 2^(exponent of t) truncated to binary32, by integer operations (et: the exponent bits of t's high
+// word): 0 below 2^-100, 2^100 above.
+__device__ __forceinline__ float over_f32(double x, unsigned et) {
+  const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+  const int ex = (int)((hi & 0x7ff00000u) - et) >> 20;
+  const unsigned man = __funnelshift_l(lo, hi, 3) & 0x7fffffu, sg = hi & 0x80000000u;
+  return ex < -100 ? 0.0f : __uint_as_float(sg | (ex > 100 ? 227u << 23 : ((unsigned)(ex + 127) << 23 | man)));
+}
+
+// The next point of the screened probes (any point does; only the number of probes depends on it, so it
+// is placed in binary32, relative to t): the pole model's root, near t by one fixed-point step of
+// dt = F / (1 - dpsi p / (p + dt)), p = t - E, else from its quadratic x^2 - A x + dpsi p^2 = 0,
+// x = p + dt, A = a0 + psi + dpsi p - E; F = a0 - t + Psi.
 __device__ __forceinline__ double model_point(double t, double F, double psi, double dpsi, double E, double a0) {
-  const double p = __dsub_rn(t, E);
-  const double d0 = quot_approx(F, __dsub_rn(1.0, dpsi));
-  if (!(p > 0.0) || !(p <= 1.0e300)) return __dadd_rn(t, d0);
-  const double pd = __dadd_rn(p, d0);
-  // |d0| < p / 4 (by the exponents)
-  if (((__double2hiint(d0) & 0x7fffffff) >> 20) + 2 < (__double2hiint(p) >> 20))
-    return __dadd_rn(t, quot_approx(F, __fma_rn(-dpsi, quot_approx(p, pd), 1.0)));
-  const double s = __dmul_rn(__dmul_rn(-dpsi, p), p);
-  const double A = __dsub_rn(__dadd_rn(a0, __fma_rn(dpsi, p, psi)), E);
-  const double disc = root(__fma_rn(A, A, __dmul_rn(4.0, s)));
-  return __dadd_rn(E, is_negative(A) ? quot_approx(__dadd_rn(s, s), __dsub_rn(disc, A))
-                                     : __dmul_rn(0.5, __dadd_rn(A, disc)));
+  const unsigned et = (unsigned)__double2hiint(t) & 0x7ff00000u;
+  const float f = over_f32(F, et), s = -over_f32(dpsi, 0x3ff00000u), p = over_f32(__dsub_rn(t, E), et);
+  const float d0 = __fmul_rn(f, rcp_approx_f32(1.0f + s));
+  float dt = d0;
+  if (p > 0.0f && p < 0x1p99f) {
+    if (4.0f * fabsf(d0) < p) {
+      dt = __fmul_rn(f, rcp_approx_f32(__fmaf_rn(s, __fmul_rn(p, rcp_approx_f32(p + d0)), 1.0f)));
+    } else {
+      const float A = over_f32(__dadd_rn(a0, psi), et) - over_f32(E, et) - s * p;
+      const float c = s * p * p, disc = __fsqrt_rn(__fmaf_rn(A, A, 4.0f * c));
+      dt = (A < 0.0f ? 2.0f * c * rcp_approx_f32(disc - A) : 0.5f * (A + disc)) - p;
+    }
+  }
+  return __fma_rn((double)dt, __hiloint2double((int)et, 0), t);
 }
 
 // No screen: every step evaluates phi.
