@@ -468,16 +468,17 @@ __global__ void k_deflate(Prob pb, Ws w) {
 // (solve_pole checks the near end, so a wrong sign of a rounded F costs steps, not accuracy).
 // ---------------------------------------------------------------------------------
 // ---------------------------------------------------------------------------------
-// One eigenvector row by a warp (Eq. (eigenvecAi)): x_j = zeta_j / ((d_j - sigma) - mu) (for a
+// One eigenvector row by a lane group (Eq. (eigenvecAi)): x_j = zeta_j / ((d_j - sigma) - mu) (for a
 // pole shift d_i, x_i = -zeta_i / mu), ||x|| with a scaled fallback when the plain sum of squares
 // over- or underflows.  With vr the row v = x / ||x|| is written there: the first pass stores
 // x_j as it forms them (pairs of components from a 16-byte aligned position, lane 0 taking an
 // unaligned first and an unpaired last one) and the second rescales them in place.  Returns
 // *nrm = ||x|| scale and *scale (v_j = x_j scale / *nrm).
 // ---------------------------------------------------------------------------------
+template <int L>
 __device__ __forceinline__ void row_values(const double* __restrict__ d, const double* __restrict__ z, int n,
-                                           double s, double m, double* __restrict__ vr, int lane, double* nrm_out,
-                                           double* scale_out) {
+                                           double s, double m, double* __restrict__ vr, int lane, unsigned gm,
+                                           double* nrm_out, double* scale_out, double* c_out) {
   const bool store = vr != nullptr;
   double q = 0.0;
   bool bad = false;
@@ -485,7 +486,7 @@ __device__ __forceinline__ void row_values(const double* __restrict__ d, const d
   const int npair = (store && kVecPairs) ? (n - j0) >> 1 : 0;
   const int jtail = j0 + 2 * npair;
   if (store && kVecPairs) {
-    for (int t = lane; t < npair; t += 32) {
+    for (int t = lane; t < npair; t += L) {
       const int j = j0 + 2 * t;
       const double den0 = __dsub_rn(__dsub_rn(d[j], s), m), den1 = __dsub_rn(__dsub_rn(d[j + 1], s), m);
       double2 x;
@@ -509,7 +510,7 @@ __device__ __forceinline__ void row_values(const double* __restrict__ d, const d
       }
     }
   } else {
-    for (int j = lane; j < n; j += 32) {
+    for (int j = lane; j < n; j += L) {
       const double den = __dsub_rn(__dsub_rn(d[j], s), m);
       const double x = __dmul_rn(z[j], rcp_nr(den));
       bad |= !rcp_in_range(den);
@@ -517,30 +518,31 @@ __device__ __forceinline__ void row_values(const double* __restrict__ d, const d
       q = __fma_rn(x, x, q);
     }
   }
-  q = group_sum<32>(q, FULL);
-  bad = group_any<32>(bad, FULL);
+  q = group_sum<L>(q, gm);
+  bad = group_any<L>(bad, gm);
   double scale = 1.0;                  // v_j = x_j * scale / sqrt(q)
   bool rewrite = false;                // the stored x_j are not usable: write v_j from scratch
   if (bad || !(q < 1e300) || !(q > 1e-280)) {
     double mx = 0.0;
-    for (int j = lane; j < n; j += 32) mx = fmax(mx, fabs(__dmul_rn(z[j], rcp(__dsub_rn(__dsub_rn(d[j], s), m)))));
-    mx = group_max<32>(mx, FULL);
+    for (int j = lane; j < n; j += L) mx = fmax(mx, fabs(__dmul_rn(z[j], rcp(__dsub_rn(__dsub_rn(d[j], s), m)))));
+    mx = group_max<L>(mx, gm);
     scale = 1.0 / mx;
     q = 0.0;
-    for (int j = lane; j < n; j += 32) {
+    for (int j = lane; j < n; j += L) {
       double x = __dmul_rn(z[j], rcp(__dsub_rn(__dsub_rn(d[j], s), m))) * scale;
       q = __fma_rn(x, x, q);
     }
-    q = group_sum<32>(q, FULL);
+    q = group_sum<L>(q, gm);
     rewrite = true;
   }
   const double nrm = sqrt(q);          // ||x|| * scale
   const double c = scale / nrm;
   *nrm_out = nrm;
   *scale_out = scale;
+  *c_out = c;
   if (!store) return;
   if (!rewrite && kVecPairs) {
-    for (int t = lane; t < npair; t += 32) {
+    for (int t = lane; t < npair; t += L) {
       const int j = j0 + 2 * t;
       double2 x = *reinterpret_cast<const double2*>(vr + j);
       x.x = __dmul_rn(x.x, c);
@@ -552,9 +554,9 @@ __device__ __forceinline__ void row_values(const double* __restrict__ d, const d
       if (jtail < n) vr[n - 1] = __dmul_rn(vr[n - 1], c);
     }
   } else if (!rewrite) {
-    for (int j = lane; j < n; j += 32) vr[j] = __dmul_rn(vr[j], c);
+    for (int j = lane; j < n; j += L) vr[j] = __dmul_rn(vr[j], c);
   } else {
-    for (int j = lane; j < n; j += 32) vr[j] = __dmul_rn(z[j], rcp(__dsub_rn(__dsub_rn(d[j], s), m))) * c;
+    for (int j = lane; j < n; j += L) vr[j] = __dmul_rn(z[j], rcp(__dsub_rn(__dsub_rn(d[j], s), m))) * c;
   }
 }
 
@@ -562,8 +564,8 @@ __device__ __forceinline__ void row_values(const double* __restrict__ d, const d
 // and its record: the pair it was formed from, ||x|| scale and the scale.
 __device__ __noinline__ void tail_row(const double* __restrict__ d, const double* __restrict__ z, int n, double s,
                                       double m, double* __restrict__ vr, int lane, double* __restrict__ rec) {
-  double nrm, scale;
-  row_values(d, z, n, s, m, vr, lane, &nrm, &scale);
+  double nrm, scale, c;
+  row_values<32>(d, z, n, s, m, vr, lane, FULL, &nrm, &scale, &c);
   if (lane == 0) {
     rec[0] = s;
     rec[1] = m;
@@ -1024,7 +1026,7 @@ __global__ void k_defl_positions(Prob pb, Ws w) {
 }
 
 // ---------------------------------------------------------------------------------
-// k_vectors: one warp per eigenvalue row.  x_j = zeta_j / ((d_j - sigma) - mu) (for a
+// k_vectors: one lane group per eigenvalue row.  x_j = zeta_j / ((d_j - sigma) - mu) (for a
 // pole shift d_i this is Eq. (eigenvecAi), with x_i = -zeta_i / mu), ||x|| with a
 // scaled fallback when the plain sum of squares over- or underflows, v = x / ||x||.
 // Each x_j is evaluated once: the first pass stores it in the output row while summing
@@ -1047,7 +1049,7 @@ __device__ __forceinline__ void pair_outputs(const Prob& pb, const Ws& w, int p,
   const int ea = w.pexp[2 * p], eb = w.pexp[2 * p + 1];
   const double lz = w.lamz[g];
   const double lam = isnan(lz) ? __dadd_rn(s, m) : lz;
-  const double xn = nrm / scale;
+  const double xn = scale == 1.0 ? nrm : nrm / scale;
   pb.lambda[base + row] = scalbn(lam, ea);
   if (pb.sigma) pb.sigma[base + row] = scalbn(s, ea);
   if (pb.mu) pb.mu[base + row] = scalbn(m, ea);
@@ -1059,11 +1061,15 @@ __device__ __forceinline__ void pair_outputs(const Prob& pb, const Ws& w, int p,
   if (out) atomicOr(w.status, ST_RANGE);
 }
 
+// A lane group of L lanes per row: a batch of small problems takes 8 or 16, since the row's scalar work
+// (norm, scaling, the pair's outputs) costs a warp as much for one row as for four.
+template <int L>
 __global__ void __launch_bounds__(256) k_vectors(Prob pb, Ws w) {
   if (*w.status & ST_FATAL) return;
-  const int lane = threadIdx.x & 31;
-  const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  const int lane = threadIdx.x & (L - 1);
+  const unsigned gm = group_mask<L>();
+  const int64_t wid = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / L;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) / L;
   for (int64_t g = wid; g < pb.total; g += nw) {
     const int p = p_owner(pb, w, g);
     if (w.pst[p] & PT_TRIVIAL) continue;
@@ -1088,15 +1094,14 @@ __global__ void __launch_bounds__(256) k_vectors(Prob pb, Ws w) {
       }
     }
     // without deflation the row is written with its norm; a deflated row is written below
-    double nrm, scale;
-    row_values(d, z, n, s, m, defl ? nullptr : vr, lane, &nrm, &scale);
-    const double c = scale / nrm;
+    double nrm, scale, c;
+    row_values<L>(d, z, n, s, m, defl ? nullptr : vr, lane, gm, &nrm, &scale, &c);
     if (lane == 0) {
       pair_outputs(pb, w, p, g, base, k, row, d, s, m, nrm, scale, c);
       if (vr) atomicAdd(&w.counters[C_VECROWS], 1u);
     }
     if (!vr || !defl) continue;
-    for (int qq = lane; qq < nfull; qq += 32) {
+    for (int qq = lane; qq < nfull; qq += L) {
       int sj = w.src[base + qq];
       double v = 0.0;
       if (sj >= 0) v = w.coef[base + qq] * (__dmul_rn(z[sj], rcp(__dsub_rn(__dsub_rn(d[sj], s), m))) * c);
@@ -1366,7 +1371,9 @@ static dpr1_status run_table(const Prob& pb, void* workspace, size_t wbytes, con
   int64_t vg = (pb.total + 7) / 8;
   if (vg > sms * 16) vg = sms * 16;
   if (vg < 1) vg = 1;
-  k_vectors<<<(int)vg, 256, 0, st>>>(pb, w);
+  if (pb.P > 1 && avg_n <= 128) k_vectors<8><<<(int)vg, 256, 0, st>>>(pb, w);
+  else if (pb.P > 1 && avg_n <= 512) k_vectors<16><<<(int)vg, 256, 0, st>>>(pb, w);
+  else k_vectors<32><<<(int)vg, 256, 0, st>>>(pb, w);
   record(o, 3, st);
   k_defl_rows<<<(int)vg, 256, 0, st>>>(pb, w);
   k_trivial<<<(int)vg, 256, 0, st>>>(pb, w);
