@@ -823,14 +823,16 @@ __global__ void k_arrow_zero_detect(int n, const double* __restrict__ d, ArrowWs
   }
 }
 
-__global__ void k_arrow_zero_solve(int n, const double* __restrict__ d, ArrowWs w, int cap, bool fast) {
+__global__ void __launch_bounds__(256) k_arrow_zero_solve(int n, const double* __restrict__ d, ArrowWs w, int cap,
+                                                          bool fast) {
   if (*w.status & ST_FATAL_A) return;
   const double alpha = w.scal[0];
   const int nz = (int)w.counters[C_ZERO_N];
-  const int lane = threadIdx.x & 31;
-  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int t = wid; t < nz; t += nw) {
+  // a block-wide lane group per candidate, in one of the solve kernel's buffers where it has them (one
+  // warp without them took about 0.5 ms of a 2.4 ms call at n = 2300)
+  double* const Ds = (w.terms && blockIdx.x < w.term_slots && n <= w.term_n)
+                         ? w.terms + 4 * (int64_t)blockIdx.x * w.term_n : nullptr;
+  for (int t = blockIdx.x; t < nz; t += gridDim.x) {
     const int k = w.zlist[t];
     // the poles next to 0: the first negative pole and the one before it (no pole is zero)
     int lo = 0, hi = n;
@@ -841,16 +843,15 @@ __global__ void k_arrow_zero_solve(int n, const double* __restrict__ d, ArrowWs 
     }
     bool ok;
     int st;
-    const double lam0 = solve_nonpole_arrow<32>(d, w.zl, w.zz, n, alpha, 0.0, lo - 1, lo < n ? lo : -1, cap, fast,
-                                                lane, FULL, &ok, &st);
-    if (lane == 0) {
+    const double lam0 = solve_nonpole_arrow<256>(d, w.zl, w.zz, n, alpha, 0.0, lo - 1, lo < n ? lo : -1, cap, fast,
+                                                 threadIdx.x, FULL, &ok, &st, Ds, Ds ? Ds + n : nullptr);
+    if (threadIdx.x == 0) {
       w.lamz[k] = lam0;
       atomicAdd(&w.counters[C_EVAL_FIX], (unsigned)st);
       if (!ok) atomicOr(w.status, ST_NOT_CONVERGED);
     }
   }
 }
-
 
 // Rows v_k = [x; -1] / ||.|| (one warp per row), lambda, sigma, mu, ||[x; -1]||.  A row the solve
 // kernel's tail wrote (arrow_row_values, the same arithmetic) is kept when its record holds the
@@ -1044,7 +1045,7 @@ dpr1_status dpr1_arrow_eig(int64_t n, const double* d, const double* z, double a
   const int fg = (int)(n + 1 < (int64_t)sms * AH_FIX_BLOCKS_PER_SM ? n + 1 : (int64_t)sms * AH_FIX_BLOCKS_PER_SM);
   k_arrow_fix<AH_FIX_THREADS><<<fg, AH_FIX_THREADS, 0, st>>>((int)n, ds, w, o.T_Knu, o.cap, o.fast, o.screen);
   k_arrow_zero_detect<<<kg, 256, 0, st>>>((int)n, ds, w, o.T_zero);
-  k_arrow_zero_solve<<<1, 128, 0, st>>>((int)n, ds, w, o.cap, o.fast);
+  k_arrow_zero_solve<<<2, 256, 0, st>>>((int)n, ds, w, o.cap, o.fast);
   int64_t vg = (n + 1 + 7) / 8;
   if (vg > sms * 16) vg = sms * 16;
   k_arrow_vectors<<<(int)vg, 256, 0, st>>>((int)n, ds, zs, w, lambda, Vt, ldv, sigma, mu, xnorm);

@@ -921,8 +921,7 @@ __global__ void __launch_bounds__(L > 256 ? L : 256) k_fix(Prob pb, Ws w, double
 // T_zero |lambda| < min(|lambda - d_k|, |lambda - d_{k-1}|), when no pole of the problem
 // is zero: lambda = 1/nu, nu the extreme eigenvalue of A^{-1} = D^{-1} + gamma D^{-1} z z^T D^{-1}
 // (Eq. (gamma)) -- the non-pole solve with sigma = 0.  k_zero_detect marks candidates
-// (the paper notes there is at most one per problem); k_zero_solve handles them one warp
-// each.  lamz[g] = NaN means "not recomputed".
+// (the paper notes there is at most one per problem); k_zero_solve handles them.  lamz[g] = NaN means "not recomputed".
 // ---------------------------------------------------------------------------------
 __global__ void k_zero_detect(Prob pb, Ws w, double T_zero) {
   if (*w.status & ST_FATAL) return;
@@ -946,13 +945,15 @@ __global__ void k_zero_detect(Prob pb, Ws w, double T_zero) {
   }
 }
 
-__global__ void k_zero_solve(Prob pb, Ws w, int cap, bool fast) {
+// A lane group of L threads (one per block) takes a candidate, in one of k_solve's buffers where it has
+// them.  There are few candidates, so the time is one solve's latency: a block-wide group for problems
+// of mean order above 200, a warp below, whose reductions need no barrier.
+template <int L>
+__global__ void __launch_bounds__(L) k_zero_solve(Prob pb, Ws w, int cap, bool fast) {
   if (*w.status & ST_FATAL) return;
   const int nz = (int)w.counters[C_ZERO_N];
-  const int lane = threadIdx.x & 31;
-  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  for (int t = wid; t < nz; t += nw) {
+  double* const Dbuf = (w.terms && blockIdx.x < w.term_slots) ? w.terms + 4 * (int64_t)blockIdx.x * w.term_n : nullptr;
+  for (int t = blockIdx.x; t < nz; t += gridDim.x) {
     const int64_t g = w.zlist[t];
     const int p = p_owner(pb, w, g);
     const int64_t base = p_base(pb, p);
@@ -967,10 +968,11 @@ __global__ void k_zero_solve(Prob pb, Ws w, int cap, bool fast) {
     }
     const int below = lo < n ? lo : -1;
     const int above = lo - 1;
+    double* const Ds = (Dbuf && n <= w.term_n) ? Dbuf : nullptr;
     bool ok;
-    double lam0 = solve_nonpole<32>(d, w.zl + base, w.zz + base, n, w.prho[p], 0.0, above, below, cap, fast, lane,
-                                    FULL, &ok);
-    if (lane == 0) {
+    double lam0 = solve_nonpole<L, false, true>(d, w.zl + base, w.zz + base, n, w.prho[p], 0.0, above, below, cap, fast,
+                                                threadIdx.x, FULL, &ok, nullptr, Ds, Ds ? Ds + n : nullptr);
+    if (threadIdx.x == 0) {
       w.lamz[g] = lam0;
       if (!ok) atomicOr(w.status, ST_NOT_CONVERGED);
     }
@@ -1366,7 +1368,9 @@ static dpr1_status run_table(const Prob& pb, void* workspace, size_t wbytes, con
   else if (L == 16) launch_solve_fix<16>(pb, w, o, grid, warps, avg_n, st);
   else launch_solve_fix<32>(pb, w, o, grid, warps, avg_n, st);
   k_zero_detect<<<sgrid, 256, 0, st>>>(pb, w, o.T_zero);
-  k_zero_solve<<<4, 128, 0, st>>>(pb, w, o.cap, o.fast);
+  const int zg = pb.P < 2 * sms ? (int)pb.P : 2 * sms;   // at most one candidate per problem
+  if (avg_n > 200) k_zero_solve<256><<<zg > 0 ? zg : 1, 256, 0, st>>>(pb, w, o.cap, o.fast);
+  else k_zero_solve<32><<<zg > 0 ? zg : 1, 32, 0, st>>>(pb, w, o.cap, o.fast);
   k_defl_positions<<<sgrid, 256, 0, st>>>(pb, w);
   int64_t vg = (pb.total + 7) / 8;
   if (vg > sms * 16) vg = sms * 16;
