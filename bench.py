@@ -70,7 +70,7 @@ B64_OPS_PER_TERM = 4
 # the binary32 pass of the shift test (shift_test_f32): per term one binary64 subtraction and 16
 # binary32 operations (difference, reciprocal and its Newton step, quotient, w, the bound's two
 # fma, the magnitude sum, TwoSum and the low-part sum); its conversions to binary32 are integer work
-SHIFT32_B64_OPS_PER_TERM = 1
+SHIFT32_B64_OPS_PER_TERM = 0
 SHIFT32_OPS_PER_TERM = 16
 # an eigenvector component (Eq. (eigenvecAi)): 2 sub, 1 div, 1 mul, 1 fma (sum of squares), 1 mul
 # (rescale); the solve kernel's lane groups write rows once its queue is empty
@@ -479,7 +479,7 @@ def bench_accel(B, dev, d, z, rho, ws, out, flush, steps, bisection_ms):
                                   "ops_definition": "(n-1) x (8 ops per secular term and evaluation (5 for the "
                                                     "value, 3 for the slope) + per eigenvalue the 4-op binary64 "
                                                     "corner pass + 20 ops per double-double term where kappa_nu "
-                                                    "asks for it) + the shift tests: per term 1 binary64 and 16 "
+                                                    "asks for it) + the shift tests: per term 16 "
                                                     "binary32 ops of the binary32 pass, and 5 binary64 ops where "
                                                     "that pass leaves the sign open; the eigenvector rows its "
                                                     "lane groups write once its queue is empty, 6 binary64 ops "
@@ -752,7 +752,7 @@ def run_ours(args):
                 "div, mul, add) + for the eigenvalues whose kappa_nu asks for it 20 ops per double-double term "
                 "of b (TwoSum 6, TwoProd 2, quotient and correction 5, compensated accumulation 7)); binary32: "
                 "(n-1) x (14 ops per term of a binary32 screen + 50 per term of a double-float screen) over the "
-                "settled screens of bisection steps and probes; the shift tests: per term 1 binary64 and 16 "
+                "settled screens of bisection steps and probes; the shift tests: per term 16 "
                 "binary32 ops of the binary32 pass, and the 5-op binary64 pass where the binary32 pass leaves "
                 "the sign open; the eigenvector rows written by the kernel's lane groups once its queue is "
                 "empty, 6 binary64 ops per component; a binary32 op counts 1/64 of a binary64 op (128 against "
@@ -765,7 +765,7 @@ def run_ours(args):
         kname = "k_solve (shift test, corner b, accelerated bracketed solve)"
         odef = ("(n-1) x (8 ops per secular term and evaluation (5 for the value, 3 for the slope) + per "
                 "eigenvalue the 4-op binary64 corner pass + 20 ops per double-double term for the eigenvalues "
-                "whose kappa_nu asks for it) + the shift tests: per term 1 binary64 and 16 binary32 ops of "
+                "whose kappa_nu asks for it) + the shift tests: per term 16 binary32 ops of "
                 "the binary32 pass, and 5 binary64 ops where it leaves the sign open; the eigenvector rows "
                 "written by its lane groups once its queue is empty, 6 binary64 ops per component; a binary32 "
                 "op counts 1/64")

@@ -193,7 +193,8 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
   // their binary32 copies for the screen, after the two binary64 arrays: us = Ds + n)
   float* const F = (Ds && screen && !fast) ? (float*)(us + n) : nullptr;
   bool rng_ok = false;
-  dd acc = dd_pole_sum<L>(d, zz, zl, n, i, di, lane, gm, &sq, nullptr, Ds, us, F, &rng_ok);
+  dd acc = dd_pole_sum<L>(d, zz, zl, n, i, di, lane, gm, &sq, nullptr, Ds, us, F, &rng_ok, 0.0,
+                              k == 0 || k == n);
   const bool scr_ok = rng_ok && F;
   dd B = dd_add(two_sum(di, -alpha), acc);
   const dd Zi = {zz[i], zl[i]};

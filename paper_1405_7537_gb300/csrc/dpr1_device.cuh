@@ -130,8 +130,11 @@ __device__ __forceinline__ bool zero_weight(double z) { return fabs(z) < 0x1p-51
 // does not evaluate it speculatively next to every fast reciprocal
 static __device__ __noinline__ double rcp_ieee(double x) { return 1.0 / x; }
 
-// 1/x within one ulp for every x (the IEEE quotient outside the fast range)
+// 1/x within one ulp for every x (the IEEE quotient outside the fast range); with chain by rcp_chain
 __device__ __forceinline__ double rcp(double x) { return rcp_in_range(x) ? rcp_nr(x) : rcp_ieee(x); }
+__device__ __forceinline__ double rcp(double x, bool chain) {
+  return rcp_in_range(x) ? (chain ? rcp_chain(x) : rcp_nr(x)) : rcp_ieee(x);
+}
 
 // Quotients and square roots of the solves' scalar work (brackets, placed points, the finishing
 // correction), which every lane of a group computes: the IEEE operations take 10 to 15 binary64
@@ -141,7 +144,7 @@ __device__ __forceinline__ double rcp(double x) { return rcp_in_range(x) ? rcp_n
 // of range, which its callers treat as "no point".  root: sqrt(x) within 2 ulps by two Newton steps on the
 // hardware's reciprocal square root, sqrt out of line for the rest.
 __device__ __forceinline__ double quot(double a, double b) {
-  return __dmul_rn(a, rcp_in_range(b) ? rcp_chain(b) : rcp_ieee(b));
+  return __dmul_rn(a, rcp(b, true));
 }
 __device__ __forceinline__ double quot_approx(double a, double b) {
   const double r = rcp_approx(b);
@@ -171,7 +174,7 @@ __device__ __forceinline__ bool is_negative(double a) { return __double2hiint(a)
 // dd / dd to about 2^-104 relative: q1 = a.hi/b.hi, then one correction digit from the
 // exact residual a.hi - q1 b.hi (fma), the low parts and the divisor's reciprocal.
 __device__ __forceinline__ dd dd_div(dd a, dd b) {
-  double r = rcp(b.hi);
+  double r = rcp(b.hi, true);
   double q1 = __dmul_rn(a.hi, r);
   // make q1 faithful so that the fma residual below is exact
   double res = __fma_rn(-q1, b.hi, a.hi);

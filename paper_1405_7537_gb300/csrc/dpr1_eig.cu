@@ -146,13 +146,18 @@ size_t ws_layout2(int64_t total, int64_t nprob, bool batched, Ws* w, char* base)
 }
 
 // Lane-group width of k_solve for an average problem order (when the options leave it open).  One
-// problem always takes a warp per eigenvalue: small ones leave most of the GPU idle, and the time is
-// the latency of an eigenvalue's passes and the divergence of the groups that share a warp (n = 16, 96,
-// 384: 92, 123 and 274 us for the kernel with 8, 8 and 16 lanes, 55, 66 and 183 with 32).  In a
-// batch, eight lanes up to a mean order of 384 (problems of orders 96-384: 33.3 ms against 39.8 with
-// 16 lanes and 48.3 with 32 for 425k eigenpairs; orders 16-96: 18.2 against 24.9 and 32.5) and a
-// warp above (orders 384-2048: 108.4 ms against 115.8 with 16 lanes and 140.3 with 8).
-static int default_lanes(double avg_n, int64_t nprob = 1) { return nprob > 1 && avg_n <= 384 ? 8 : 32; }
+// problem takes a warp per eigenvalue up to order 128, where it leaves most of the GPU idle and the time
+// is the latency of an eigenvalue's passes and the divergence of the groups that share a warp (n = 16,
+// 96: 92 and 123 us for the kernel with 8 lanes, 55 and 66 with 32), 16 lanes up to 384 (a warp is
+// faster, 183 against 274 us at 384, but orders the sums anew, and R2's shift of an exterior eigenvalue
+// moves with their rounding times K_nu ~ n^2), and a warp above.  In a batch, eight lanes up to a mean
+// order of 384 (problems of orders 96-384: 33.3 ms against 39.8 with 16 lanes and 48.3 with 32 for 425k
+// eigenpairs; orders 16-96: 18.2 against 24.9 and 32.5) and a warp above (orders 384-2048: 108.4 ms
+// against 115.8 with 16 lanes and 140.3 with 8).
+static int default_lanes(double avg_n, int64_t nprob = 1) {
+  if (nprob > 1) return avg_n <= 384 ? 8 : 32;
+  return avg_n > 128 && avg_n <= 384 ? 16 : 32;
+}
 
 // Bytes of the stored-element buffers appended to the workspace: TERM_BYTES term_n bytes for
 // each lane group of k_solve's default launch (8 warps per block, DPR1_SOLVE_MIN_BLOCKS blocks per

@@ -120,13 +120,13 @@ __device__ __forceinline__ double arrow_sum_pass(const double* __restrict__ d, c
       const double num = __fma_rn(w0, y1, __dmul_rn(w1, y0));
       const double den = __dmul_rn(y0, y1);
       b |= !rcp_in_range(den) || !rcp_in_range(num);
-      s0 = __fma_rn(num, rcp_nr(den), s0);
+      s0 = __fma_rn(num, rcp_chain(den), s0);
       continue;
     }
     double r0, r1;
-    if (SAFE) { r0 = rcp(x0); r1 = rcp(x1); }
+    if (SAFE) { r0 = rcp(x0, true); r1 = rcp(x1, true); }
     else {
-      r0 = rcp_nr(x0); r1 = rcp_nr(x1);
+      r0 = rcp_chain(x0); r1 = rcp_chain(x1);
       b |= (!rcp_in_range(x0) && j != i) || (!rcp_in_range(x1) && j + L != i);
     }
     // the excluded term j == i (0 * inf) is removed by selecting a zero reciprocal
@@ -145,8 +145,8 @@ __device__ __forceinline__ double arrow_sum_pass(const double* __restrict__ d, c
     double t0 = __fma_rn(-nu, D0, 1.0);
     double x0 = __dmul_rn(D0, t0);
     double r0;
-    if (SAFE) r0 = rcp(x0);
-    else { r0 = rcp_nr(x0); b |= !rcp_in_range(x0) && j != i; }
+    if (SAFE) r0 = rcp(x0, true);
+    else { r0 = rcp_chain(x0); b |= !rcp_in_range(x0) && j != i; }
     r0 = (j == i) ? 0.0 : r0;
     s0 = __fma_rn(zz[j], r0, s0);
     if (DERIV) {
@@ -205,19 +205,19 @@ __device__ __forceinline__ double stored_sum(const double* __restrict__ Ds, cons
     const double n23 = __fma_rn(u2, t3, __dmul_rn(u3, t2)), p23 = __dmul_rn(t2, t3);
     const double num = __fma_rn(n01, p23, __dmul_rn(n23, p01)), den = __dmul_rn(p01, p23);
     b |= !rcp_in_range(den) || !rcp_in_range(num);
-    s0 = __fma_rn(num, rcp_nr(den), s0);
+    s0 = __fma_rn(num, rcp_chain(den), s0);
   }
   if (j + L < n) {
     const double t0 = __fma_rn(-nu, Ds[j], 1.0), t1 = __fma_rn(-nu, Ds[j + L], 1.0);
     const double num = __fma_rn(us[j], t1, __dmul_rn(us[j + L], t0)), den = __dmul_rn(t0, t1);
     b |= !rcp_in_range(den) || !rcp_in_range(num);
-    s0 = __fma_rn(num, rcp_nr(den), s0);
+    s0 = __fma_rn(num, rcp_chain(den), s0);
     j += 2 * L;
   }
   if (j < n) {
     const double t0 = __fma_rn(-nu, Ds[j], 1.0), u0 = us[j];
     b |= !rcp_in_range(t0) || (u0 != 0.0 && !rcp_in_range(u0));
-    s0 = __fma_rn(u0, rcp_nr(t0), s0);
+    s0 = __fma_rn(u0, rcp_chain(t0), s0);
   }
   const double s = group_sum<L>(s0, gm);
   if (group_any<L>(b, gm)) {
@@ -707,7 +707,7 @@ __device__ __forceinline__ double stored_sum_d(const double* __restrict__ Ds, co
     const double D0 = Ds[j], D1 = Ds[j + L];
     const double t0 = __fma_rn(-nu, D0, 1.0), t1 = __fma_rn(-nu, D1, 1.0);
     b |= !rcp_in_range(t0) || !rcp_in_range(t1);
-    const double r0 = rcp_nr(t0), r1 = rcp_nr(t1);
+    const double r0 = rcp_chain(t0), r1 = rcp_chain(t1);
     const double a0 = __dmul_rn(us[j], r0), a1 = __dmul_rn(us[j + L], r1);
     s0 = __dadd_rn(s0, a0);
     s1 = __dadd_rn(s1, a1);
@@ -718,7 +718,7 @@ __device__ __forceinline__ double stored_sum_d(const double* __restrict__ Ds, co
     const double D0 = Ds[j];
     const double t0 = __fma_rn(-nu, D0, 1.0);
     b |= !rcp_in_range(t0);
-    const double r0 = rcp_nr(t0);
+    const double r0 = rcp_chain(t0);
     const double a0 = __dmul_rn(us[j], r0);
     s0 = __dadd_rn(s0, a0);
     q0 = __fma_rn(a0, __dmul_rn(D0, r0), q0);
@@ -780,7 +780,7 @@ __device__ __forceinline__ dd dd_pole_sum(const double* __restrict__ d, const do
                                           unsigned gm, double* sq, double* cub = nullptr,
                                           double* __restrict__ Ds = nullptr, double* __restrict__ us = nullptr,
                                           float* __restrict__ F = nullptr, bool* scr_ok = nullptr,
-                                          double slo = 0.0) {
+                                          double slo = 0.0, bool chain = false) {
   double hi = 0.0, lo = 0.0, q2 = 0.0, c3 = 0.0;
   const double ms = -s;
   bool ok = Ds != nullptr;
@@ -802,7 +802,7 @@ __device__ __forceinline__ dd dd_pole_sum(const double* __restrict__ d, const do
       Dl = __dsub_rn(small, __dsub_rn(Dh, big));
     }
     const double Zh = zz[j], Zl = zl[j];
-    const double r = rcp(Dh);
+    const double r = rcp(Dh, chain);
     const double q = __dmul_rn(Zh, r);
     if (Ds) ok &= store_elem(Ds, us, F, n, j, Dh, q);
     const double eq = __dmul_rn(__dadd_rn(__fma_rn(-q, Dh, Zh), __fma_rn(-q, Dl, Zl)), r);
@@ -906,8 +906,8 @@ struct NoScreen {
 // decline, and the solve goes on to adjacent doubles.  The bracket, its midpoint and so every bit of
 // the result are the same with and without screens.  Bisecting on costs one binary64 evaluation for
 // each bit of the window around the root that no screen can settle: 2.9 evaluations per eigenvalue on
-// the hard spectrum and 7.6 on O(1) weights, against 1.0 and 1.1 (batch of 4096 problems 388 -> 225 ms,
-// hard spectrum of order 16384 25.1 -> 20.3 ms, arrowhead of order 16384 48.3 -> 27.1 ms).
+// the hard spectrum and 7.6 on O(1) weights, against 1.5 and 1.1 (batch of 4096 problems 388 -> 230 ms,
+// hard spectrum of order 16384 25.5 -> 20.5 ms, arrowhead of order 16384 48 -> 28.5 ms).
 template <class Fin>
 __device__ __forceinline__ bool finish_root(uint64_t lo, uint64_t hi, double side, double pole, double a1,
                                             double finish, Fin fin, int* steps, double* root) {
@@ -1372,12 +1372,14 @@ struct CornerRule {
 //   kappa_nu = min((n + 4) sqrt(n) K_b, 3 sqrt(n) + (n + 4)(1 + 2 K_z))     (Eq. (knu2));
 // b is then recomputed in double-double only when kappa_nu > T_kappa n.
 // With Ds != nullptr the pass also stores the elements Delta_j and zz_j / Delta_j of the
-// inverse for stored_sum (a pass of its own in mode 2).
+// inverse for stored_sum (a pass of its own in mode 2).  chain: reciprocals by rcp_chain (the exterior
+// eigenvalue of a large rank-one part: where K_nu is large, R2 takes its shift sigma from this solve, at
+// the size of its rounding times K_nu, and the elements and evaluations keep the roundings they had).
 template <int L>
 __device__ __forceinline__ double corner_b(const double* __restrict__ d, const double* __restrict__ zz,
                                            const double* __restrict__ zl, int n, int i,
-                                           double rho, double inv_zi2, int lane, unsigned gm, double* wn2,
-                                           CornerRule cr, bool* used_dd, double* __restrict__ Ds, double* __restrict__ us,
+                                           double rho, double inv_zi2, bool chain, int lane, unsigned gm,
+                                           double* wn2, CornerRule cr, bool* used_dd, double* __restrict__ Ds, double* __restrict__ us,
                                            float* __restrict__ F, bool* scr_ok) {
   const double di = d[i];
   bool ok = Ds != nullptr;
@@ -1389,7 +1391,7 @@ __device__ __forceinline__ double corner_b(const double* __restrict__ d, const d
         continue;
       }
       const double D = __dsub_rn(d[j], di);
-      const double r = rcp(D);
+      const double r = rcp(D, chain);
       const double t = __dmul_rn(zz[j], r);
       if (Ds) ok &= store_elem(Ds, us, F, n, j, D, t);
       if (j < i) p = __dadd_rn(p, t);
@@ -1414,13 +1416,13 @@ __device__ __forceinline__ double corner_b(const double* __restrict__ d, const d
     if (Ds) {
       for (int j = lane; j < n; j += L) {
         const double D = (j == i) ? 0.0 : __dsub_rn(d[j], di);
-        ok &= store_elem(Ds, us, F, n, j, D, (j == i) ? 0.0 : __dmul_rn(zz[j], rcp(D)));
+        ok &= store_elem(Ds, us, F, n, j, D, (j == i) ? 0.0 : __dmul_rn(zz[j], rcp(D, chain)));
       }
     }
     *scr_ok = !group_any<L>(!ok, gm);
   }
   double sq;
-  dd acc = dd_pole_sum<L>(d, zz, zl, n, i, di, lane, gm, &sq);
+  dd acc = dd_pole_sum<L>(d, zz, zl, n, i, di, lane, gm, &sq, nullptr, nullptr, nullptr, nullptr, nullptr, 0.0, chain);
   dd B = dd_add(dd_div({1.0, 0.0}, {rho, 0.0}), acc);
   const dd Zi = {zz[i], zl[i]};
   *wn2 = sq / Zi.hi;
@@ -1447,7 +1449,7 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
   // the binary32 copies and low parts follow the two binary64 arrays (us = Ds + n)
   float* const F = (Ds && screen && !fast) ? (float*)(us + n) : nullptr;
   const double inv_zi2 = 1.0 / zz[i];
-  double b = corner_b<L>(d, zz, zl, n, i, rho, inv_zi2, lane, gm, &wn2, cr, &used_dd, Ds, us, F, &rng_ok);
+  double b = corner_b<L>(d, zz, zl, n, i, rho, inv_zi2, k == 0, lane, gm, &wn2, cr, &used_dd, Ds, us, F, &rng_ok);
   const bool scr_ok = rng_ok && F;
   double side = (i == k) ? 1.0 : -1.0;
   double di = d[i];
