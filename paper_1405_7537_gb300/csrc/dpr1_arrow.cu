@@ -173,6 +173,23 @@ __global__ void k_arrow_check(int n, const double* __restrict__ d, const double*
   if ((threadIdx.x & 31) == 0 && zp) atomicOr(status + 1, zp);
 }
 
+// The corner's pass of the two exterior eigenvalues with rcp_chain's reciprocals (as corner_chain)
+struct PoleSum {
+  dd sum;
+  double sq;
+  bool ok;
+};
+template <int L>
+__device__ __noinline__ PoleSum pole_sum_chain(const double* __restrict__ d, const double* __restrict__ zz,
+                                               const double* __restrict__ zl, int n, int i, double di, int lane,
+                                               unsigned gm, double* __restrict__ Ds, double* __restrict__ us,
+                                               float* __restrict__ F) {
+  PoleSum c;
+  c.ok = false;
+  c.sum = dd_pole_sum<L, false, true>(d, zz, zl, n, i, di, lane, gm, &c.sq, nullptr, Ds, us, F, &c.ok);
+  return c;
+}
+
 // Extreme eigenvalue nu of (A - d_i I)^{-1} on the side of eigenvalue k (rightmost when
 // i == k, leftmost when i == k - 1); [alo, ahi] an estimate of the bracket of |nu|.
 template <int L, bool NI = false>
@@ -193,8 +210,15 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
   // their binary32 copies for the screen, after the two binary64 arrays: us = Ds + n)
   float* const F = (Ds && screen && !fast) ? (float*)(us + n) : nullptr;
   bool rng_ok = false;
-  dd acc = dd_pole_sum<L>(d, zz, zl, n, i, di, lane, gm, &sq, nullptr, Ds, us, F, &rng_ok, 0.0,
-                              k == 0 || k == n);
+  dd acc;
+  if (k == 0 || k == n) {
+    const PoleSum c = pole_sum_chain<L>(d, zz, zl, n, i, di, lane, gm, Ds, us, F);
+    acc = c.sum;
+    sq = c.sq;
+    rng_ok = c.ok;
+  } else {
+    acc = dd_pole_sum<L>(d, zz, zl, n, i, di, lane, gm, &sq, nullptr, Ds, us, F, &rng_ok);
+  }
   const bool scr_ok = rng_ok && F;
   dd B = dd_add(two_sum(di, -alpha), acc);
   const dd Zi = {zz[i], zl[i]};

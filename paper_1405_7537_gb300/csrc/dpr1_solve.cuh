@@ -774,13 +774,13 @@ __device__ __forceinline__ double shift_sum(const double* __restrict__ d, const 
 // (store_elem), and *scr_ok tells whether they lie in the screens' range.
 // With OFS the shift is s + slo in double the working precision: the difference is formed by
 // shift_diff and the stored element is its binary64 rounding (elem_diff).
-template <int L, bool OFS = false>
+template <int L, bool OFS = false, bool CHAIN = false>
 __device__ __forceinline__ dd dd_pole_sum(const double* __restrict__ d, const double* __restrict__ zz,
                                           const double* __restrict__ zl, int n, int skip, double s, int lane,
                                           unsigned gm, double* sq, double* cub = nullptr,
                                           double* __restrict__ Ds = nullptr, double* __restrict__ us = nullptr,
                                           float* __restrict__ F = nullptr, bool* scr_ok = nullptr,
-                                          double slo = 0.0, bool chain = false) {
+                                          double slo = 0.0) {
   double hi = 0.0, lo = 0.0, q2 = 0.0, c3 = 0.0;
   const double ms = -s;
   bool ok = Ds != nullptr;
@@ -802,7 +802,7 @@ __device__ __forceinline__ dd dd_pole_sum(const double* __restrict__ d, const do
       Dl = __dsub_rn(small, __dsub_rn(Dh, big));
     }
     const double Zh = zz[j], Zl = zl[j];
-    const double r = rcp(Dh, chain);
+    const double r = rcp(Dh, CHAIN);
     const double q = __dmul_rn(Zh, r);
     if (Ds) ok &= store_elem(Ds, us, F, n, j, Dh, q);
     const double eq = __dmul_rn(__dadd_rn(__fma_rn(-q, Dh, Zh), __fma_rn(-q, Dl, Zl)), r);
@@ -1372,14 +1372,14 @@ struct CornerRule {
 //   kappa_nu = min((n + 4) sqrt(n) K_b, 3 sqrt(n) + (n + 4)(1 + 2 K_z))     (Eq. (knu2));
 // b is then recomputed in double-double only when kappa_nu > T_kappa n.
 // With Ds != nullptr the pass also stores the elements Delta_j and zz_j / Delta_j of the
-// inverse for stored_sum (a pass of its own in mode 2).  chain: reciprocals by rcp_chain (the exterior
+// inverse for stored_sum (a pass of its own in mode 2).  CHAIN: reciprocals by rcp_chain (the exterior
 // eigenvalue of a large rank-one part: where K_nu is large, R2 takes its shift sigma from this solve, at
 // the size of its rounding times K_nu, and the elements and evaluations keep the roundings they had).
-template <int L>
+template <int L, bool CHAIN>
 __device__ __forceinline__ double corner_b(const double* __restrict__ d, const double* __restrict__ zz,
                                            const double* __restrict__ zl, int n, int i,
-                                           double rho, double inv_zi2, bool chain, int lane, unsigned gm,
-                                           double* wn2, CornerRule cr, bool* used_dd, double* __restrict__ Ds, double* __restrict__ us,
+                                           double rho, double inv_zi2, int lane, unsigned gm, double* wn2,
+                                           CornerRule cr, bool* used_dd, double* __restrict__ Ds, double* __restrict__ us,
                                            float* __restrict__ F, bool* scr_ok) {
   const double di = d[i];
   bool ok = Ds != nullptr;
@@ -1391,7 +1391,7 @@ __device__ __forceinline__ double corner_b(const double* __restrict__ d, const d
         continue;
       }
       const double D = __dsub_rn(d[j], di);
-      const double r = rcp(D, chain);
+      const double r = rcp(D, CHAIN);
       const double t = __dmul_rn(zz[j], r);
       if (Ds) ok &= store_elem(Ds, us, F, n, j, D, t);
       if (j < i) p = __dadd_rn(p, t);
@@ -1416,17 +1416,34 @@ __device__ __forceinline__ double corner_b(const double* __restrict__ d, const d
     if (Ds) {
       for (int j = lane; j < n; j += L) {
         const double D = (j == i) ? 0.0 : __dsub_rn(d[j], di);
-        ok &= store_elem(Ds, us, F, n, j, D, (j == i) ? 0.0 : __dmul_rn(zz[j], rcp(D, chain)));
+        ok &= store_elem(Ds, us, F, n, j, D, (j == i) ? 0.0 : __dmul_rn(zz[j], rcp(D, CHAIN)));
       }
     }
     *scr_ok = !group_any<L>(!ok, gm);
   }
   double sq;
-  dd acc = dd_pole_sum<L>(d, zz, zl, n, i, di, lane, gm, &sq, nullptr, nullptr, nullptr, nullptr, nullptr, 0.0, chain);
+  dd acc = dd_pole_sum<L, false, CHAIN>(d, zz, zl, n, i, di, lane, gm, &sq);
   dd B = dd_add(dd_div({1.0, 0.0}, {rho, 0.0}), acc);
   const dd Zi = {zz[i], zl[i]};
   *wn2 = sq / Zi.hi;
   return dd_to_double(dd_div(B, Zi));
+}
+
+// The chain form out of line: one solve per problem takes it, and inlined next to the other it crowds
+// the registers of both.
+struct Corner {
+  double b, wn2;
+  bool dd, ok;
+};
+template <int L>
+__device__ __noinline__ Corner corner_chain(const double* __restrict__ d, const double* __restrict__ zz,
+                                            const double* __restrict__ zl, int n, int i, double rho, double inv_zi2,
+                                            int lane, unsigned gm, CornerRule cr, double* __restrict__ Ds,
+                                            double* __restrict__ us, float* __restrict__ F) {
+  Corner c;
+  c.ok = false;
+  c.b = corner_b<L, true>(d, zz, zl, n, i, rho, inv_zi2, lane, gm, &c.wn2, cr, &c.dd, Ds, us, F, &c.ok);
+  return c;
 }
 
 // Brackets of |nu| from the shift test (see the derivation in k_solve's comment).  Ds, us: the
@@ -1449,7 +1466,16 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
   // the binary32 copies and low parts follow the two binary64 arrays (us = Ds + n)
   float* const F = (Ds && screen && !fast) ? (float*)(us + n) : nullptr;
   const double inv_zi2 = 1.0 / zz[i];
-  double b = corner_b<L>(d, zz, zl, n, i, rho, inv_zi2, k == 0, lane, gm, &wn2, cr, &used_dd, Ds, us, F, &rng_ok);
+  double b;
+  if (k == 0) {
+    const Corner c = corner_chain<L>(d, zz, zl, n, i, rho, inv_zi2, lane, gm, cr, Ds, us, F);
+    b = c.b;
+    wn2 = c.wn2;
+    used_dd = c.dd;
+    rng_ok = c.ok;
+  } else {
+    b = corner_b<L, false>(d, zz, zl, n, i, rho, inv_zi2, lane, gm, &wn2, cr, &used_dd, Ds, us, F, &rng_ok);
+  }
   const bool scr_ok = rng_ok && F;
   double side = (i == k) ? 1.0 : -1.0;
   double di = d[i];
