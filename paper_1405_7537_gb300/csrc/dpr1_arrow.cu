@@ -173,59 +173,38 @@ __global__ void k_arrow_check(int n, const double* __restrict__ d, const double*
   if ((threadIdx.x & 31) == 0 && zp) atomicOr(status + 1, zp);
 }
 
-// The corner's pass of the two exterior eigenvalues with rcp_chain's reciprocals (as corner_chain)
-struct PoleSum {
-  dd sum;
-  double sq;
-  bool ok;
-};
-template <int L>
-__device__ __noinline__ PoleSum pole_sum_chain(const double* __restrict__ d, const double* __restrict__ zz,
-                                               const double* __restrict__ zl, int n, int i, double di, int lane,
-                                               unsigned gm, double* __restrict__ Ds, double* __restrict__ us,
-                                               float* __restrict__ F) {
-  PoleSum c;
-  c.ok = false;
-  c.sum = dd_pole_sum<L, false, true>(d, zz, zl, n, i, di, lane, gm, &c.sq, nullptr, Ds, us, F, &c.ok);
-  return c;
-}
-
 // Extreme eigenvalue nu of (A - d_i I)^{-1} on the side of eigenvalue k (rightmost when
 // i == k, leftmost when i == k - 1); [alo, ahi] an estimate of the bracket of |nu|.
-template <int L, bool NI = false>
+// FIRST, check and *ill: as solve_pole.
+template <int L, bool NI = false, bool FIRST = false>
 __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const double* __restrict__ zl,
                                        const double* __restrict__ zz, int n, double alpha, int k, int i, double alo,
                                        double ahi, int cap, bool fast, int lane, unsigned gm,
                                        double* __restrict__ Ds = nullptr, double* __restrict__ us = nullptr,
-                                       bool screen = false) {
+                                       bool screen = false, bool check = false) {
   PoleResult r;
   r.screened = 0;
   r.screened_near = 0;
   r.screened_df = 0;
   r.inferred = 0;
   r.probes = 0;
+  r.steps = 0;
   double sq;
   const double di = d[i];
   // the corner's pass also stores the elements of the inverse when the group has a buffer (and
   // their binary32 copies for the screen, after the two binary64 arrays: us = Ds + n)
   float* const F = (Ds && screen && !fast) ? (float*)(us + n) : nullptr;
   bool rng_ok = false;
-  dd acc;
-  if (k == 0 || k == n) {
-    const PoleSum c = pole_sum_chain<L>(d, zz, zl, n, i, di, lane, gm, Ds, us, F);
-    acc = c.sum;
-    sq = c.sq;
-    rng_ok = c.ok;
-  } else {
-    acc = dd_pole_sum<L>(d, zz, zl, n, i, di, lane, gm, &sq, nullptr, Ds, us, F, &rng_ok);
-  }
+  float qa = 0.0f;
+  dd acc = dd_pole_sum<L, false, FIRST>(d, zz, zl, n, i, di, lane, gm, &sq, nullptr, Ds, us, F, &rng_ok, 0.0,
+                                        FIRST ? nullptr : &qa);
   const bool scr_ok = rng_ok && F;
   dd B = dd_add(two_sum(di, -alpha), acc);
   const dd Zi = {zz[i], zl[i]};
   const double b = dd_to_double(dd_div(B, Zi));
   const double inv = 1.0 / zz[i];
   const double wn2 = sq / Zi.hi + inv;          // squared border: w_j (j != i) and 1/zeta_i
-  const double wn = root(wn2);
+  const double wn = root_t<FIRST>(wn2);
   const double side = (i == k) ? 1.0 : -1.0;
   double floor, E;
   // the caller's [alo, ahi] rests on the shift test (or the 2 x 2 interlacing bounds) and is
@@ -235,35 +214,36 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
   ahi = INFINITY;
   if (side > 0) {
     // largest pole of g: the nearest pole above d_i (or, for i = 0, the farthest below), or 0
-    const double dmax = (i > 0) ? quot(1.0, d[i - 1] - di) : (n > 1 ? quot(1.0, d[n - 1] - di) : -INFINITY);
+    const double dmax = (i > 0) ? quot_t<FIRST>(1.0, d[i - 1] - di) : (n > 1 ? quot_t<FIRST>(1.0, d[n - 1] - di) : -INFINITY);
     const double pmax = fmax(dmax, 0.0);
     floor = pmax;
     E = pmax;
     alo = fmax(alo, b);
     ahi = fmin(ahi, fmax(b, pmax) + wn);
-    if (b > pmax) ahi = fmin(ahi, b + quot(wn2, b - pmax));
+    if (b > pmax) ahi = fmin(ahi, b + quot_t<FIRST>(wn2, b - pmax));
     // smallest pole: the nearest delta_j below d_i (or the farthest above), or 0
-    const double dmin = (i + 1 < n) ? quot(1.0, d[i + 1] - di) : (n > 1 ? quot(1.0, d[0] - di) : INFINITY);
-    quad_bracket(b, fmin(dmin, 0.0), pmax, wn2, &alo, &ahi);
+    const double dmin = (i + 1 < n) ? quot_t<FIRST>(1.0, d[i + 1] - di) : (n > 1 ? quot_t<FIRST>(1.0, d[0] - di) : INFINITY);
+    quad_bracket<FIRST>(b, fmin(dmin, 0.0), pmax, wn2, &alo, &ahi);
   } else {
-    const double dmin = (i + 1 < n) ? quot(1.0, d[i + 1] - di) : (n > 1 ? quot(1.0, d[0] - di) : INFINITY);
+    const double dmin = (i + 1 < n) ? quot_t<FIRST>(1.0, d[i + 1] - di) : (n > 1 ? quot_t<FIRST>(1.0, d[0] - di) : INFINITY);
     const double pmin = fmin(dmin, 0.0);
     floor = -pmin;
     E = -pmin;
     alo = fmax(alo, -b);
     ahi = fmin(ahi, -fmin(b, pmin) + wn);
-    if (b < pmin) ahi = fmin(ahi, -b + quot(wn2, pmin - b));
-    const double dmx = (i > 0) ? quot(1.0, d[i - 1] - di) : (n > 1 ? quot(1.0, d[n - 1] - di) : -INFINITY);
-    quad_bracket(-b, -fmax(dmx, 0.0), -pmin, wn2, &alo, &ahi);
+    if (b < pmin) ahi = fmin(ahi, -b + quot_t<FIRST>(wn2, pmin - b));
+    const double dmx = (i > 0) ? quot_t<FIRST>(1.0, d[i - 1] - di) : (n > 1 ? quot_t<FIRST>(1.0, d[n - 1] - di) : -INFINITY);
+    quad_bracket<FIRST>(-b, -fmax(dmx, 0.0), -pmin, wn2, &alo, &ahi);
   }
   const bool eager_lo = alo_in > alo, eager_hi = ahi_in < ahi;
   alo = fmax(alo, alo_in) * (1.0 - 0x1p-48);
   ahi = fmin(ahi, ahi_in) * (1.0 + 0x1p-48);
+  const double size = fabs(b) + inv * (double)qa;       // and inv / |nu| of the pole at 0
   bool ok;
   int steps = 0;
   double nu;
   // the finishing step (as in solve_pole, with the pole at 0)
-  const double finish = rng_ok && inv < 0x1p100 ? (k == 0 || k == n ? kFinishCondExt : kFinishCond) : 0.0;
+  const double finish = !FIRST && rng_ok && inv < 0x1p100 ? kFinishCond : 0.0;
   const float cf = (float)inv;
   auto fin = [&](double v, double* Fv, double* s, double* mag) -> bool {
     double S;
@@ -277,6 +257,13 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
     *s = (double)q + ex / v;
     return isfinite(q);
   };
+  r.ill = false;
+  if (!FIRST && check && (!rng_ok || size + inv / alo > kIllCond * alo)) {
+    double Fv, s = 0.0, m;
+    r.ill = !rng_ok || !fin(side * ahi, &Fv, &s, &m) || size + inv / alo > kIllCond * alo * (1.0 + s);
+    r.steps = rng_ok;
+    if (r.ill) return r;
+  }
   uint64_t blo, bhi;
   start_bracket(&floor, alo, ahi, &blo, &bhi);
   if (fast && finish > 0.0 && bhi - blo <= kFinishWidth &&
@@ -360,8 +347,19 @@ __device__ PoleResult solve_pole_arrow(const double* __restrict__ d, const doubl
   r.b = b;
   r.ok = ok;
   r.dd = true;
-  r.steps = steps;
+  r.steps += steps;
   return r;
+}
+
+// As solve_pole_first (the bracket of an exterior eigenvalue comes from the caller).
+template <int L>
+__device__ __noinline__ PoleResult solve_pole_arrow_first(const double* __restrict__ d, const double* __restrict__ zl,
+                                                          const double* __restrict__ zz, int n, double alpha, int k,
+                                                          int i, double alo, double ahi, int cap, bool fast, int lane,
+                                                          unsigned gm, double* __restrict__ Ds,
+                                                          double* __restrict__ us, bool screen) {
+  if (k > 0 && k < n) alo = 1.0 / __dmul_rn(__dsub_rn(d[k - 1], d[k]), 0.5);
+  return solve_pole_arrow<L, true, true>(d, zl, zz, n, alpha, k, i, alo, ahi, cap, fast, lane, gm, Ds, us, screen);
 }
 
 // One eigenvector row v = [x; -1] / ||.|| by a warp: x_j = zeta_j / ((d_j - sigma) - mu), ||[x; -1]||
@@ -432,7 +430,7 @@ __device__ __noinline__ void arrow_tail_row(const double* __restrict__ d, const 
 // k_arrow_vectors writes the others and rewrites a row whose pair the remedies changed.
 template <int L>
 __global__ void __launch_bounds__(256, DPR1_SOLVE_MIN_BLOCKS) k_arrow_solve(int n, const double* __restrict__ d,
-                                                     const double* __restrict__ z, ArrowWs w, int cap,
+                                                     const double* __restrict__ z, ArrowWs w, int gpw, int cap,
                                                      bool fast, bool screen, double* __restrict__ Vt, int64_t ldv) {
   if (*w.status & ST_FATAL_A) return;
   const double alpha = w.scal[0];       // d, z and alpha are the normalised copies
@@ -440,7 +438,9 @@ __global__ void __launch_bounds__(256, DPR1_SOLVE_MIN_BLOCKS) k_arrow_solve(int 
   const unsigned gm = group_mask<L>();
   const int leader = (threadIdx.x & 31) & ~(L - 1);
   const double* __restrict__ zz = w.zz;
-  const int64_t grp = (int64_t)blockIdx.x * (blockDim.x / L) + threadIdx.x / L;
+  const int sub = (threadIdx.x & 31) / L;
+  if (sub >= gpw) return;               // gpw lane groups of each warp work
+  const int64_t grp = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * gpw + sub;
   double* const Dbuf = (w.terms && grp < w.term_slots && n <= w.term_n) ? w.terms + 4 * grp * w.term_n : nullptr;
   for (;;) {
     long long gl = 0;
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(256, DPR1_SOLVE_MIN_BLOCKS) k_arrow_solve(int 
       shift32 = sf != 0;
       if (!shift32) {
         for (int j = lane; j < n; j += L) {
-          const double t = __dmul_rn(zz[j], rcp(__dsub_rn(__dsub_rn(d[j], dk), tau)));
+          const double t = __dmul_rn(zz[j], rcp_c(__dsub_rn(__dsub_rn(d[j], dk), tau)));
           if (j < k) sp = __dadd_rn(sp, t);
           else sn = __dadd_rn(sn, t);
         }
@@ -528,8 +528,18 @@ __global__ void __launch_bounds__(256, DPR1_SOLVE_MIN_BLOCKS) k_arrow_solve(int 
       }
       if (!(ahi > alo)) ahi = INFINITY;
     }
-    PoleResult pr = solve_pole_arrow<L, true>(d, w.zl, zz, n, alpha, k, i, alo, ahi, cap, fast, lane, gm, Dbuf,
-                                        Dbuf ? Dbuf + n : nullptr, screen);
+    double* const us = Dbuf ? Dbuf + n : nullptr;
+    PoleResult pr;
+    pr.steps = 0;
+    pr.ill = k == 0 || k == n || !Dbuf;   // as k_solve
+    if (!pr.ill)
+      pr = solve_pole_arrow<L, true>(d, w.zl, zz, n, alpha, k, i, alo, ahi, cap, fast, lane, gm, Dbuf, us, screen,
+                                     true);
+    if (pr.ill) {
+      const int checked = pr.steps;
+      pr = solve_pole_arrow_first<L>(d, w.zl, zz, n, alpha, k, i, alo, ahi, cap, fast, lane, gm, Dbuf, us, screen);
+      pr.steps += checked;
+    }
     if (lane == 0) {
       if (pr.screened) atomicAdd(&w.counters[C_SCREEN], (unsigned)pr.screened);
       if (pr.screened_near) atomicAdd(&w.counters[C_SCREEN_NEAR], (unsigned)pr.screened_near);
@@ -939,12 +949,11 @@ __global__ void k_arrow_one(double alpha, double* lambda, double* Vt, double* si
   if (Vt) Vt[0] = -1.0;
 }
 
-// lane groups of the solve kernel's default launch and of the remedies kernel
-// (a warp per eigenvalue, as for one problem D + rho z z^T)
-static int arrow_lanes(int64_t) { return 32; }
+// lane groups of the solve kernel's default launch (as default_lanes for one problem D + rho z z^T)
+static int arrow_lanes(int64_t n) { return n <= 96 ? 8 : (n <= 384 ? 16 : 32); }
 
-static int64_t arrow_groups(int64_t n, int L, int warps, int bps) {
-  const int groups_per_block = (32 * warps) / L;
+static int64_t arrow_groups(int64_t n, int gpw, int warps, int bps) {
+  const int groups_per_block = gpw * warps;
   int64_t want = (n + 1 + groups_per_block - 1) / groups_per_block;
   int64_t grid = (int64_t)sm_count() * bps;
   if (want < grid) grid = want > 0 ? want : 1;
@@ -966,7 +975,7 @@ static size_t arrow_tail_bytes(int64_t n) {
 static size_t arrow_term_bytes(int64_t n) {
   if (n <= 0) return 0;
   const int64_t tn = (n + 31) & ~(int64_t)31;
-  return (size_t)arrow_groups(n, arrow_lanes(n), 8, DPR1_SOLVE_MIN_BLOCKS) * TERM_BYTES * (size_t)tn +
+  return (size_t)arrow_groups(n, 32 / arrow_lanes(n), 8, DPR1_SOLVE_MIN_BLOCKS) * TERM_BYTES * (size_t)tn +
          arrow_tail_bytes(n);
 }
 
@@ -976,16 +985,18 @@ static size_t arrow_term_bytes(int64_t n) {
 template <int L>
 static dpr1_status launch_arrow(int n, const double* d, const double* z, ArrowWs* w, const Options& o, char* tail,
                                 size_t tb, double* Vt, int64_t ldv, cudaStream_t st) {
+  // one lane group per warp by default, also where it is narrower (as run_table's gpw)
+  const int gpw = o.lanes ? 32 / L : 1;
   // fewer lane groups than 8-warp blocks on every SM hold: blocks of fewer warps, one per SM
   int warps = o.warps;
   if (o.warps_auto && o.bps_auto) {
-    const int64_t w_need = (((int64_t)n + 1) * L + 32 * (int64_t)sm_count() - 1) / (32 * (int64_t)sm_count());
+    const int64_t w_need = ((int64_t)n + 1 + (int64_t)gpw * sm_count() - 1) / ((int64_t)gpw * sm_count());
     // no more lane groups (a last block rounds up) than the default launch's, which have buffers
-    const int64_t most = ((int64_t)n + 1 + 256 / L - 1) / (256 / L) * (256 / L);
+    const int64_t most = ((int64_t)n + 1 + 8 * gpw - 1) / (8 * gpw) * (8 * gpw);
     warps = w_need < 8 ? (int)w_need : 8;
-    while (warps < 8 && ((int64_t)n + 32 * warps / L) / (32 * warps / L) * (32 * warps / L) > most) warps++;
+    while (warps < 8 && ((int64_t)n + warps * gpw) / (warps * gpw) * (warps * gpw) > most) warps++;
   }
-  const int groups_per_block = (32 * warps) / L;
+  const int groups_per_block = gpw * warps;
   int64_t want = ((int64_t)n + 1 + groups_per_block - 1) / groups_per_block;
   int grid = sm_count() * o.bps;
   if (want < grid) grid = (int)(want > 0 ? want : 1);
@@ -994,7 +1005,7 @@ static dpr1_status launch_arrow(int n, const double* d, const double* z, ArrowWs
     // formed the same way whichever group takes an eigenvalue)
     const int64_t tn = ((int64_t)n + 31) & ~(int64_t)31;
     const int64_t slots = (int64_t)(tb / (TERM_BYTES * (size_t)tn));
-    const int64_t need = arrow_groups(n, L, warps, o.bps);
+    const int64_t need = arrow_groups(n, gpw, warps, o.bps);
     if (slots >= need) {
       w->terms = (double*)tail;
       w->term_n = tn;
@@ -1012,7 +1023,7 @@ static dpr1_status launch_arrow(int n, const double* d, const double* z, ArrowWs
       }
     }
   }
-  k_arrow_solve<L><<<grid, 32 * warps, 0, st>>>(n, d, z, *w, o.cap, o.fast, o.screen, Vt, ldv);
+  k_arrow_solve<L><<<grid, 32 * warps, 0, st>>>(n, d, z, *w, gpw, o.cap, o.fast, o.screen, Vt, ldv);
   return DPR1_OK;
 }
 

@@ -130,11 +130,9 @@ __device__ __forceinline__ bool zero_weight(double z) { return fabs(z) < 0x1p-51
 // does not evaluate it speculatively next to every fast reciprocal
 static __device__ __noinline__ double rcp_ieee(double x) { return 1.0 / x; }
 
-// 1/x within one ulp for every x (the IEEE quotient outside the fast range); with chain by rcp_chain
+// 1/x within one ulp for every x (the IEEE quotient outside the fast range), by rcp_nr or by rcp_chain
 __device__ __forceinline__ double rcp(double x) { return rcp_in_range(x) ? rcp_nr(x) : rcp_ieee(x); }
-__device__ __forceinline__ double rcp(double x, bool chain) {
-  return rcp_in_range(x) ? (chain ? rcp_chain(x) : rcp_nr(x)) : rcp_ieee(x);
-}
+__device__ __forceinline__ double rcp_c(double x) { return rcp_in_range(x) ? rcp_chain(x) : rcp_ieee(x); }
 
 // Quotients and square roots of the solves' scalar work (brackets, placed points, the finishing
 // correction), which every lane of a group computes: the IEEE operations take 10 to 15 binary64
@@ -144,7 +142,7 @@ __device__ __forceinline__ double rcp(double x, bool chain) {
 // of range, which its callers treat as "no point".  root: sqrt(x) within 2 ulps by two Newton steps on the
 // hardware's reciprocal square root, sqrt out of line for the rest.
 __device__ __forceinline__ double quot(double a, double b) {
-  return __dmul_rn(a, rcp(b, true));
+  return __dmul_rn(a, rcp_c(b));
 }
 __device__ __forceinline__ double quot_approx(double a, double b) {
   const double r = rcp_approx(b);
@@ -161,6 +159,15 @@ __device__ __forceinline__ double root(double x) {
   return __fma_rn(__fma_rn(-s, s, x), h, s);
 }
 
+// The same operations in a chosen form: IEEE (quotient, square root, reciprocals by rcp_chain) or the
+// cheaper ones above.
+template <bool IEEE>
+__device__ __forceinline__ double rcp_t(double x) { return IEEE ? rcp_c(x) : rcp(x); }
+template <bool IEEE>
+__device__ __forceinline__ double quot_t(double a, double b) { return IEEE ? a / b : quot(a, b); }
+template <bool IEEE>
+__device__ __forceinline__ double root_t(double x) { return IEEE ? sqrt(x) : root(x); }
+
 // order of the magnitudes of doubles as integers (a binary64 comparison takes the binary64 pipe):
 // |a| > |b|, false when a is NaN or infinite
 __device__ __forceinline__ bool mag_greater(double a, double b) {
@@ -174,7 +181,7 @@ __device__ __forceinline__ bool is_negative(double a) { return __double2hiint(a)
 // dd / dd to about 2^-104 relative: q1 = a.hi/b.hi, then one correction digit from the
 // exact residual a.hi - q1 b.hi (fma), the low parts and the divisor's reciprocal.
 __device__ __forceinline__ dd dd_div(dd a, dd b) {
-  double r = rcp(b.hi, true);
+  double r = rcp_c(b.hi);
   double q1 = __dmul_rn(a.hi, r);
   // make q1 faithful so that the fma residual below is exact
   double res = __fma_rn(-q1, b.hi, a.hi);

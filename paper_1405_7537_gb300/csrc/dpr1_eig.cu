@@ -145,18 +145,19 @@ size_t ws_layout2(int64_t total, int64_t nprob, bool batched, Ws* w, char* base)
   return off;
 }
 
-// Lane-group width of k_solve for an average problem order (when the options leave it open).  One
-// problem takes a warp per eigenvalue up to order 128, where it leaves most of the GPU idle and the time
-// is the latency of an eigenvalue's passes and the divergence of the groups that share a warp (n = 16,
-// 96: 92 and 123 us for the kernel with 8 lanes, 55 and 66 with 32), 16 lanes up to 384 (a warp is
-// faster, 183 against 274 us at 384, but orders the sums anew, and R2's shift of an exterior eigenvalue
-// moves with their rounding times K_nu ~ n^2), and a warp above.  In a batch, eight lanes up to a mean
-// order of 384 (problems of orders 96-384: 33.3 ms against 39.8 with 16 lanes and 48.3 with 32 for 425k
-// eigenpairs; orders 16-96: 18.2 against 24.9 and 32.5) and a warp above (orders 384-2048: 108.4 ms
-// against 115.8 with 16 lanes and 140.3 with 8).
+// Lane-group width of k_solve for an average problem order (when the options leave it open).  The width
+// orders the sums, and the shift of an eigenvalue that R2 takes keeps their rounding (solve_pole), so one
+// problem's widths are part of the result: 8 lanes to order 96, 16 to 384, a warp above.  Its groups take a
+// warp each all the same (gpw in run_table): groups that share a warp diverge, and one small problem leaves
+// the GPU idle (whole call, us, packed and a warp each: n = 200 280 and 264, n = 384 395 and 386).
+// With 32 lanes n = 96 takes 180 us against 226: the exterior eigenvalue's
+// solve, 8 lanes wide, is the longest.  In a batch, eight lanes up to a mean order of 384 (problems of
+// orders 96-384: 33.3 ms against 39.8 with 16 lanes and 48.3 with 32 for 425k eigenpairs; orders 16-96: 18.2
+// against 24.9 and 32.5, with the solver of that time, half as fast) and a warp above (orders 384-2048:
+// 108.4 ms against 115.8 with 16 lanes and 140.3 with 8).
 static int default_lanes(double avg_n, int64_t nprob = 1) {
   if (nprob > 1) return avg_n <= 384 ? 8 : 32;
-  return avg_n > 128 && avg_n <= 384 ? 16 : 32;
+  return avg_n <= 96 ? 8 : (avg_n <= 384 ? 16 : 32);
 }
 
 // Bytes of the stored-element buffers appended to the workspace: TERM_BYTES term_n bytes for
@@ -581,18 +582,24 @@ __device__ __noinline__ void tail_row(const double* __restrict__ d, const double
 
 template <int L, int MINB, bool NI>
 __global__ void __launch_bounds__(256, MINB)
-    k_solve(Prob pb, Ws w, int cap, bool fast, int dd_mode, double T_kappa, bool screen) {
+    k_solve(Prob pb, Ws w, int gpw, int cap, bool fast, int dd_mode, double T_kappa, bool screen) {
   if (*w.status & ST_FATAL) return;
   const int lane = threadIdx.x & (L - 1);
   const unsigned gm = group_mask<L>();
   const int leader = (threadIdx.x & 31) & ~(L - 1);
-  const int64_t grp = (int64_t)blockIdx.x * (blockDim.x / L) + threadIdx.x / L;
+  const int sub = (threadIdx.x & 31) / L;
+  if (sub >= gpw) return;               // gpw lane groups of each warp work (run_table)
+  const int64_t grp = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * gpw + sub;
   double* const Dbuf = (w.terms && grp < w.term_slots) ? w.terms + 4 * grp * w.term_n : nullptr;
   for (;;) {
     long long gl = 0;
     if (lane == 0) gl = (long long)atomicAdd(&w.counters64[0], 1ull);
     gl = __shfl_sync(gm, gl, leader, 32);
-    if (gl >= pb.total) {
+    // a batch's exterior eigenvalues first: they take the FIRST form (solve_pole), and the lane groups of
+    // a warp that run it share its instructions (2000 problems of orders 16-128: 4.19 ms in the elements'
+    // order, 2.97 so; 4096 of orders 16-2048: 161.6 and 159)
+    const int64_t lead = pb.P > 1 ? pb.P : 0;
+    if (gl >= pb.total + lead) {
       if constexpr (kTailRows && L == 32 && NI) {
         // the queue is empty: write the eigenvector rows of the eigenvalues solved so far (one
         // problem without deflation), sweeping all rows once in order.  A row whose eigenvalue is
@@ -631,13 +638,14 @@ __global__ void __launch_bounds__(256, MINB)
       }
       break;
     }
-    const int64_t g = gl;
-    const int p = p_owner(pb, w, g);
+    const int p = gl < lead ? (int)gl : p_owner(pb, w, gl - lead);
+    if (gl < lead && p_size(pb, p) == 0) continue;      // no element writes an empty problem's nred
     if (w.pst[p] & PT_TRIVIAL) continue;
     const int64_t base = p_base(pb, p);
+    const int64_t g = gl < lead ? base : gl - lead;
     const int n = w.nred[p];
     const int k = (int)(g - base);
-    if (k >= n) continue;
+    if (k >= n || (k == 0 && gl >= lead && lead)) continue;
     const double rho = w.prho[p];   // rho' of the normalised problem
     const double* __restrict__ d = w.dr + base;
     const double* __restrict__ zl = w.zl + base;
@@ -662,7 +670,7 @@ __global__ void __launch_bounds__(256, MINB)
       if (sf == 0) {
         for (int j = lane; j < n; j += L) {
           double den = __dsub_rn(__dsub_rn(d[j], dk), tau);
-          double t = __dmul_rn(zz[j], rcp(den));
+          double t = __dmul_rn(zz[j], rcp_c(den));
           if (j < k) sp = __dadd_rn(sp, t);
           else sn = __dadd_rn(sn, t);
         }
@@ -681,9 +689,21 @@ __global__ void __launch_bounds__(256, MINB)
       }
     }
     const bool stored = Dbuf && n <= w.term_n;
-    PoleResult pr = solve_pole<L, NI>(d, zl, zz, n, rho, k, i, alo, ahi, cap, fast, lane, gm,
-                                  CornerRule{dd_mode, T_kappa, w.pzsum[p]}, stored ? Dbuf : nullptr,
-                                  stored ? Dbuf + n : nullptr, screen);
+    const CornerRule cr{dd_mode, T_kappa, w.pzsum[p]};
+    double* const Ds = stored ? Dbuf : nullptr;
+    double* const us = stored ? Dbuf + n : nullptr;
+    PoleResult pr;
+    pr.steps = 0;
+    // the FIRST form for the exterior eigenvalue too, whose mu is of the size of rho ||z||^2, and without
+    // stored elements (no finishing step)
+    pr.ill = k == 0 || !stored;
+    if (!pr.ill)
+      pr = solve_pole<L, NI>(d, zl, zz, n, rho, k, i, alo, ahi, cap, fast, lane, gm, cr, Ds, us, screen, true);
+    if (pr.ill) {
+      const int checked = pr.steps;
+      pr = solve_pole_first<L, NI>(d, zl, zz, n, rho, k, i, alo, ahi, cap, fast, lane, gm, cr, Ds, us, screen);
+      pr.steps += checked;
+    }
     if (lane == 0) {
       if (pr.dd) atomicAdd(&w.counters[C_DD], 1u);
       if (pr.screened) atomicAdd(&w.counters[C_SCREEN], (unsigned)pr.screened);
@@ -770,7 +790,8 @@ __device__ __forceinline__ bool pole_difference_cancels(double dp, double s, dou
 //  (R1) solve at the other neighbouring pole o when K' < K, K' <= T_Knu and ratio <= T_Knu
 //       (beyond that ratio the eigenvector formula at d_o cancels); K' and the ratio come
 //       from k_classify, so the solve runs only when it is taken.
-//  (R2) otherwise shift to sigma = fl(lambda) of the first pole solution, moved into the
+//  (R2) otherwise shift to sigma = fl(lambda) of the first pole solution (in a fixed arithmetic where it
+//       is ill-conditioned: solve_pole), moved into the
 //       interlacing interval of lambda_k ((d_k, d_{k-1}); (d_0, d_0 + rho ||z||^2] for k = 0),
 //       and solve_nonpole.  Any sigma there yields lambda_k (the sign of f(sigma) picks the
 //       side), accurately once lambda_k is the eigenvalue nearest to sigma; when |mu| is not
@@ -1250,15 +1271,15 @@ static void record(const Options& o, int t, cudaStream_t st) {
 }
 
 template <int L>
-static void launch_solve_fix(const Prob& pb, const Ws& w, const Options& o, int grid, int warps, double avg_n,
+static void launch_solve_fix(const Prob& pb, const Ws& w, const Options& o, int grid, int warps, int gpw, double avg_n,
                              cudaStream_t st) {
   record(o, 0, st);
   if (L == 32 && avg_n > DPR1_SOLVE_LARGE_N)
-    k_solve<32, DPR1_SOLVE_MIN_BLOCKS, true><<<grid, 32 * warps, 0, st>>>(pb, w, o.cap, o.fast, o.dd_mode, o.T_kappa,
-                                                                          o.screen);
+    k_solve<32, DPR1_SOLVE_MIN_BLOCKS, true><<<grid, 32 * warps, 0, st>>>(pb, w, gpw, o.cap, o.fast, o.dd_mode,
+                                                                          o.T_kappa, o.screen);
   else
-    k_solve<L, DPR1_SOLVE_SMALL_BLOCKS, false><<<grid, 32 * warps, 0, st>>>(pb, w, o.cap, o.fast, o.dd_mode, o.T_kappa,
-                                                                           o.screen);
+    k_solve<L, DPR1_SOLVE_SMALL_BLOCKS, false><<<grid, 32 * warps, 0, st>>>(pb, w, gpw, o.cap, o.fast, o.dd_mode,
+                                                                           o.T_kappa, o.screen);
   record(o, 1, st);
   int64_t cg = (pb.total + 255) / 256;
   if (cg > sm_count() * 8) cg = sm_count() * 8;
@@ -1324,9 +1345,11 @@ static dpr1_status run_table(const Prob& pb, void* workspace, size_t wbytes, con
   // inlined; DPR1_SOLVE_LARGE_N)
   if (o.bps_auto && !(L == 32 && avg_n > DPR1_SOLVE_LARGE_N) && bps > DPR1_SOLVE_SMALL_BLOCKS)
     bps = DPR1_SOLVE_SMALL_BLOCKS;
-  const int64_t lanes_total = pb.total * L;
+  // one problem's lane groups take a warp each also where they are narrower (default_lanes); a batch, or
+  // a width from the options, fills the warps
+  const int gpw = pb.P == 1 && !o.lanes ? 1 : 32 / L;
   if (o.warps_auto) {
-    const int64_t w_need = (lanes_total + 32 * (int64_t)sms - 1) / (32 * (int64_t)sms);
+    const int64_t w_need = (pb.total + gpw * (int64_t)sms - 1) / (gpw * (int64_t)sms);
     if (w_need <= 8) {
       warps = (int)(w_need > 0 ? w_need : 1);
       if (o.bps_auto) bps = 1;
@@ -1338,7 +1361,7 @@ static dpr1_status run_table(const Prob& pb, void* workspace, size_t wbytes, con
       }
     }
   }
-  int groups_per_block = (32 * warps) / L;
+  int groups_per_block = gpw * warps;
   int64_t want_blocks = (pb.total + groups_per_block - 1) / groups_per_block;
   int grid = sms * bps;
   if (want_blocks < grid) grid = want_blocks > 0 ? (int)want_blocks : 1;
@@ -1369,9 +1392,9 @@ static dpr1_status run_table(const Prob& pb, void* workspace, size_t wbytes, con
       }
     }
   }
-  if (L == 8) launch_solve_fix<8>(pb, w, o, grid, warps, avg_n, st);
-  else if (L == 16) launch_solve_fix<16>(pb, w, o, grid, warps, avg_n, st);
-  else launch_solve_fix<32>(pb, w, o, grid, warps, avg_n, st);
+  if (L == 8) launch_solve_fix<8>(pb, w, o, grid, warps, gpw, avg_n, st);
+  else if (L == 16) launch_solve_fix<16>(pb, w, o, grid, warps, gpw, avg_n, st);
+  else launch_solve_fix<32>(pb, w, o, grid, warps, gpw, avg_n, st);
   k_zero_detect<<<sgrid, 256, 0, st>>>(pb, w, o.T_zero);
   const int zg = pb.P < 2 * sms ? (int)pb.P : 2 * sms;   // at most one candidate per problem
   if (avg_n > 200) k_zero_solve<256><<<zg > 0 ? zg : 1, 256, 0, st>>>(pb, w, o.cap, o.fast);

@@ -57,7 +57,6 @@ constexpr int kPredictSteps = DPR1_PREDICT_STEPS;
 constexpr uint64_t kPredictStop = 4;
 // width (in doubles) of the bracket at which the bisection of stored elements in range hands over to
 // the finishing step, and the largest condition (the size of F's terms over t |F'|) at which it applies
-// (kFinishCondExt for the exterior eigenvalues, whose mu is of the size of rho ||z||^2)
 #ifndef DPR1_FINISH_BITS
 #define DPR1_FINISH_BITS 16
 #endif
@@ -65,7 +64,10 @@ constexpr uint64_t kFinishWidth = 1ull << DPR1_FINISH_BITS;
 #ifndef DPR1_FINISH_COND
 #define DPR1_FINISH_COND 256.0
 #endif
-constexpr double kFinishCond = DPR1_FINISH_COND, kFinishCondExt = 4.0;
+constexpr double kFinishCond = DPR1_FINISH_COND;
+// condition of the root (the size of the corner and of the terms of the secular function over |nu| times
+// the slope) above which an eigenvalue's first solve takes solve_pole's FIRST form
+constexpr double kIllCond = 0x1p20;
 
 // ---------------------------------------------------------------------------------
 // Shifts in double the working precision (remedy R2 when no binary64 number lies between
@@ -124,7 +126,7 @@ __device__ __forceinline__ double arrow_sum_pass(const double* __restrict__ d, c
       continue;
     }
     double r0, r1;
-    if (SAFE) { r0 = rcp(x0, true); r1 = rcp(x1, true); }
+    if (SAFE) { r0 = rcp_c(x0); r1 = rcp_c(x1); }
     else {
       r0 = rcp_chain(x0); r1 = rcp_chain(x1);
       b |= (!rcp_in_range(x0) && j != i) || (!rcp_in_range(x1) && j + L != i);
@@ -145,7 +147,7 @@ __device__ __forceinline__ double arrow_sum_pass(const double* __restrict__ d, c
     double t0 = __fma_rn(-nu, D0, 1.0);
     double x0 = __dmul_rn(D0, t0);
     double r0;
-    if (SAFE) r0 = rcp(x0, true);
+    if (SAFE) r0 = rcp_c(x0);
     else { r0 = rcp_chain(x0); b |= !rcp_in_range(x0) && j != i; }
     r0 = (j == i) ? 0.0 : r0;
     s0 = __fma_rn(zz[j], r0, s0);
@@ -773,15 +775,17 @@ __device__ __forceinline__ double shift_sum(const double* __restrict__ d, const 
 // elements of the inverse that stored_sum reads; with F their binary32 copies and low parts
 // (store_elem), and *scr_ok tells whether they lie in the screens' range.
 // With OFS the shift is s + slo in double the working precision: the difference is formed by
-// shift_diff and the stored element is its binary64 rounding (elem_diff).
-template <int L, bool OFS = false, bool CHAIN = false>
+// shift_diff and the stored element is its binary64 rounding (elem_diff).  FIRST: the reciprocals'
+// form (solve_pole).  *mag: the sum of |zz_j / Dh| (binary32; for elements in the screens' range).
+template <int L, bool OFS = false, bool FIRST = true>
 __device__ __forceinline__ dd dd_pole_sum(const double* __restrict__ d, const double* __restrict__ zz,
                                           const double* __restrict__ zl, int n, int skip, double s, int lane,
                                           unsigned gm, double* sq, double* cub = nullptr,
                                           double* __restrict__ Ds = nullptr, double* __restrict__ us = nullptr,
                                           float* __restrict__ F = nullptr, bool* scr_ok = nullptr,
-                                          double slo = 0.0) {
+                                          double slo = 0.0, float* mag = nullptr) {
   double hi = 0.0, lo = 0.0, q2 = 0.0, c3 = 0.0;
+  float qa = 0.0f;
   const double ms = -s;
   bool ok = Ds != nullptr;
   for (int j = lane; j < n; j += L) {
@@ -802,8 +806,9 @@ __device__ __forceinline__ dd dd_pole_sum(const double* __restrict__ d, const do
       Dl = __dsub_rn(small, __dsub_rn(Dh, big));
     }
     const double Zh = zz[j], Zl = zl[j];
-    const double r = rcp(Dh, CHAIN);
+    const double r = rcp_t<FIRST>(Dh);
     const double q = __dmul_rn(Zh, r);
+    if (mag) qa = __fadd_rn(qa, mag_f32(q));
     if (Ds) ok &= store_elem(Ds, us, F, n, j, Dh, q);
     const double eq = __dmul_rn(__dadd_rn(__fma_rn(-q, Dh, Zh), __fma_rn(-q, Dl, Zl)), r);
     const dd t = two_sum(hi, q);
@@ -816,6 +821,7 @@ __device__ __forceinline__ dd dd_pole_sum(const double* __restrict__ d, const do
   *sq = group_sum<L>(q2, gm);
   if (cub) *cub = group_sum<L>(c3, gm);
   if (scr_ok) *scr_ok = !group_any<L>(!ok, gm);
+  if (mag) *mag = group_sum_f<L>(qa, gm);
   return group_sum_dd<L>(two_sum(hi, lo), gm);
 }
 
@@ -1321,10 +1327,11 @@ __device__ double accel_solve(Ev ev, double floor, double alo, double ahi, doubl
 
 // Larger root t of (t - B)(t - E) = W (W >= 0), evaluated without cancellation; +-inf or
 // NaN when an argument is not finite (callers then ignore the bound).
+template <bool IEEE>
 __device__ __forceinline__ double qroot(double B, double E, double W) {
   const double c = E - B;
-  const double s = root(__fma_rn(c, c, 4.0 * W));
-  const double x = is_negative(c) ? 0.5 * (s - c) : quot(2.0 * W, c + s);
+  const double s = root_t<IEEE>(__fma_rn(c, c, 4.0 * W));
+  const double x = (IEEE ? !(c > 0.0) : is_negative(c)) ? 0.5 * (s - c) : quot_t<IEEE>(2.0 * W, c + s);
   return E + x;
 }
 
@@ -1334,9 +1341,10 @@ __device__ __forceinline__ double qroot(double B, double E, double W) {
 // W / (t - Enear), and t between the larger roots of (t - B)(t - Efar) = W and
 // (t - B)(t - Enear) = W.  (The corner bound B + W / (B - Enear) is this upper bound with
 // t - Enear replaced by B - Enear.)
+template <bool IEEE>
 __device__ __forceinline__ void quad_bracket(double B, double Efar, double Enear, double W, double* alo,
                                              double* ahi) {
-  const double lo = qroot(B, Efar, W), hi = qroot(B, Enear, W);
+  const double lo = qroot<IEEE>(B, Efar, W), hi = qroot<IEEE>(B, Enear, W);
   if (finite(lo)) *alo = fmax(*alo, lo);
   if (finite(hi)) *ahi = fmin(*ahi, hi);
 }
@@ -1354,7 +1362,9 @@ struct PoleResult {
   int screened_df;     // of those, steps settled by the double-float screen
   int inferred;        // bisection steps decided by certified bounds (no evaluation)
   int probes;          // screened probes that placed those bounds
+  bool ill;            // the eigenvalue needs the FIRST form
 };
+
 
 // How the corner b is formed (Sec. 2.3): mode 1 in double the working precision when kappa_nu of
 // Eq. (knu2) exceeds T_kappa n, as Algorithm 1 does, mode 2 always; zsum = sum_j |zeta_j| of the
@@ -1372,15 +1382,14 @@ struct CornerRule {
 //   kappa_nu = min((n + 4) sqrt(n) K_b, 3 sqrt(n) + (n + 4)(1 + 2 K_z))     (Eq. (knu2));
 // b is then recomputed in double-double only when kappa_nu > T_kappa n.
 // With Ds != nullptr the pass also stores the elements Delta_j and zz_j / Delta_j of the
-// inverse for stored_sum (a pass of its own in mode 2).  CHAIN: reciprocals by rcp_chain (the exterior
-// eigenvalue of a large rank-one part: where K_nu is large, R2 takes its shift sigma from this solve, at
-// the size of its rounding times K_nu, and the elements and evaluations keep the roundings they had).
-template <int L, bool CHAIN>
+// inverse for stored_sum (a pass of its own in mode 2).  *mag: the size of the terms of the secular
+// function, (1/zeta_i^2) sum_{j != i} zeta_j^2/|d_j - d_i|.  FIRST: see solve_pole.
+template <int L, bool FIRST>
 __device__ __forceinline__ double corner_b(const double* __restrict__ d, const double* __restrict__ zz,
                                            const double* __restrict__ zl, int n, int i,
                                            double rho, double inv_zi2, int lane, unsigned gm, double* wn2,
                                            CornerRule cr, bool* used_dd, double* __restrict__ Ds, double* __restrict__ us,
-                                           float* __restrict__ F, bool* scr_ok) {
+                                           float* __restrict__ F, bool* scr_ok, double* mag) {
   const double di = d[i];
   bool ok = Ds != nullptr;
   if (cr.mode != 2) {
@@ -1391,7 +1400,7 @@ __device__ __forceinline__ double corner_b(const double* __restrict__ d, const d
         continue;
       }
       const double D = __dsub_rn(d[j], di);
-      const double r = rcp(D, CHAIN);
+      const double r = rcp_t<FIRST>(D);
       const double t = __dmul_rn(zz[j], r);
       if (Ds) ok &= store_elem(Ds, us, F, n, j, D, t);
       if (j < i) p = __dadd_rn(p, t);
@@ -1399,7 +1408,8 @@ __device__ __forceinline__ double corner_b(const double* __restrict__ d, const d
       s2 = __fma_rn(t, r, s2);
     }
     const double P = group_sum<L>(p, gm), N = group_sum<L>(q, gm);
-    *wn2 = group_sum<L>(s2, gm) * inv_zi2;
+    *wn2 = FIRST ? group_sum<L>(s2, gm) / zz[i] : group_sum<L>(s2, gm) * inv_zi2;
+    *mag = inv_zi2 * (P - N);
     const double nn = (double)n, sn = root(nn);
     const double rP = rho * P, rN = rho * N;
     const double Kb = quot((1.0 + rP) - rN, fabs((1.0 + rP) + rN));
@@ -1416,72 +1426,67 @@ __device__ __forceinline__ double corner_b(const double* __restrict__ d, const d
     if (Ds) {
       for (int j = lane; j < n; j += L) {
         const double D = (j == i) ? 0.0 : __dsub_rn(d[j], di);
-        ok &= store_elem(Ds, us, F, n, j, D, (j == i) ? 0.0 : __dmul_rn(zz[j], rcp(D, CHAIN)));
+        ok &= store_elem(Ds, us, F, n, j, D, (j == i) ? 0.0 : __dmul_rn(zz[j], rcp_t<FIRST>(D)));
       }
     }
     *scr_ok = !group_any<L>(!ok, gm);
   }
   double sq;
-  dd acc = dd_pole_sum<L, false, CHAIN>(d, zz, zl, n, i, di, lane, gm, &sq);
+  float qa;
+  dd acc = dd_pole_sum<L, false, FIRST>(d, zz, zl, n, i, di, lane, gm, &sq, nullptr, nullptr, nullptr, nullptr, nullptr,
+                                        0.0, cr.mode == 2 ? &qa : nullptr);
+  if (cr.mode == 2) *mag = inv_zi2 * (double)qa;
   dd B = dd_add(dd_div({1.0, 0.0}, {rho, 0.0}), acc);
   const dd Zi = {zz[i], zl[i]};
   *wn2 = sq / Zi.hi;
   return dd_to_double(dd_div(B, Zi));
 }
 
-// The chain form out of line: one solve per problem takes it, and inlined next to the other it crowds
-// the registers of both.
-struct Corner {
-  double b, wn2;
-  bool dd, ok;
-};
-template <int L>
-__device__ __noinline__ Corner corner_chain(const double* __restrict__ d, const double* __restrict__ zz,
-                                            const double* __restrict__ zl, int n, int i, double rho, double inv_zi2,
-                                            int lane, unsigned gm, CornerRule cr, double* __restrict__ Ds,
-                                            double* __restrict__ us, float* __restrict__ F) {
-  Corner c;
-  c.ok = false;
-  c.b = corner_b<L, true>(d, zz, zl, n, i, rho, inv_zi2, lane, gm, &c.wn2, cr, &c.dd, Ds, us, F, &c.ok);
-  return c;
-}
-
 // Brackets of |nu| from the shift test (see the derivation in k_solve's comment).  Ds, us: the
 // lane group's private buffers of n doubles each for the elements of the inverse (evaluations
 // with stored_sum), or nullptr (each evaluation forms them from d and zz).
-template <int L, bool NI = false>
+//
+// Two forms.  An ill-conditioned eigenvalue goes to R2, which shifts to the lambda found here: its
+// rounding, magnified by K_nu, is the returned sigma (and mu = lambda - sigma), although lambda and the
+// eigenvector do not depend on it.  FIRST fixes every operation that enters such a lambda (elements and
+// sums by rcp_chain, brackets by IEEE quotients and square roots, the adjacent doubles of the sign change
+// without the finishing step), so that (sigma, mu) do not move with the arithmetic of the others.  The
+// other form, for the rest, uses the seeded reciprocals, cheap quotients and the finishing step; with
+// check it returns before the solve, with *ill set, where the elements leave the screens' range or |b| and
+// the terms of the secular function may exceed kIllCond |nu| |dF/dnu|.  Psi is convex, so |dF/dnu| at the
+// upper end of the bracket, one evaluation where |b| and the terms exceed kIllCond times the lower end,
+// bounds it from below.  kIllCond = 2^20 leaves a rounding of at most about 2^-30 of mu in the others; in the
+// FIRST form are 4% to 7% of the eigenvalues of spectra with tight pairs of poles when the slope is left
+// out, and about 1% with it (eigenvalues only of order 6000: 6.2 and 4.4 ms; hard spectrum of order 16384
+// 21.2 and 18.4 ms).  As two functions: in one body with a loop the common form loses registers (batch of
+// 4096 problems 176 ms against 160).
+template <int L, bool NI = false, bool FIRST = false>
 __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __restrict__ zl,
                                  const double* __restrict__ zz, int n, double rho, int k, int i, double alo,
                                  double ahi, int cap, bool fast, int lane, unsigned gm, CornerRule cr,
                                  double* __restrict__ Ds = nullptr, double* __restrict__ us = nullptr,
-                                 bool screen = false) {
+                                 bool screen = false, bool check = false) {
   PoleResult r;
   r.screened = 0;
   r.screened_near = 0;
   r.screened_df = 0;
   r.inferred = 0;
   r.probes = 0;
+  r.steps = 0;
   double wn2;
   bool used_dd, rng_ok = false;
   // the binary32 copies and low parts follow the two binary64 arrays (us = Ds + n)
   float* const F = (Ds && screen && !fast) ? (float*)(us + n) : nullptr;
   const double inv_zi2 = 1.0 / zz[i];
-  double b;
-  if (k == 0) {
-    const Corner c = corner_chain<L>(d, zz, zl, n, i, rho, inv_zi2, lane, gm, cr, Ds, us, F);
-    b = c.b;
-    wn2 = c.wn2;
-    used_dd = c.dd;
-    rng_ok = c.ok;
-  } else {
-    b = corner_b<L, false>(d, zz, zl, n, i, rho, inv_zi2, lane, gm, &wn2, cr, &used_dd, Ds, us, F, &rng_ok);
-  }
+  double mag;
+  const double b = corner_b<L, FIRST>(d, zz, zl, n, i, rho, inv_zi2, lane, gm, &wn2, cr, &used_dd, Ds, us, F, &rng_ok,
+                                      &mag);
   const bool scr_ok = rng_ok && F;
   double side = (i == k) ? 1.0 : -1.0;
   double di = d[i];
   // Weyl: the extreme eigenvalue lies within ||w|| of max(b, max delta) (rightmost) or
   // min(b, min delta) (leftmost); Rayleigh: nu >= b (rightmost), nu <= b (leftmost).
-  double wn = root(wn2);
+  double wn = root_t<FIRST>(wn2);
   // floor: the pole of g next to the extreme eigenvalue (largest delta_j for the
   // rightmost, smallest for the leftmost), or 0 when all poles lie on the other side.
   double floor, E;   // E: the nearest pole on |nu| (the accelerated solve's model pole)
@@ -1495,26 +1500,26 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
   // pole b ~ 1/zeta_i^2 dominates and this bracket is narrow.
   if (side > 0) {
     // largest delta_j: the nearest pole above d_i, or for i = 0 the farthest pole below
-    double dmax = (i > 0) ? quot(1.0, d[i - 1] - di) : (n > 1 ? quot(1.0, d[n - 1] - di) : -INFINITY);
+    double dmax = (i > 0) ? quot_t<FIRST>(1.0, d[i - 1] - di) : (n > 1 ? quot_t<FIRST>(1.0, d[n - 1] - di) : -INFINITY);
     floor = fmax(dmax, 0.0);
     E = dmax;
     rlo = b;
     rhi = fmax(b, dmax) + wn;
-    if (b > dmax) rhi = fmin(rhi, b + quot(wn2, b - dmax));
+    if (b > dmax) rhi = fmin(rhi, b + quot_t<FIRST>(wn2, b - dmax));
     // smallest delta_j: the nearest pole below d_i, or for i = n-1 the farthest pole above
-    const double dmin = (i + 1 < n) ? quot(1.0, d[i + 1] - di) : (n > 1 ? quot(1.0, d[0] - di) : -INFINITY);
-    quad_bracket(b, dmin, dmax, wn2, &rlo, &rhi);
+    const double dmin = (i + 1 < n) ? quot_t<FIRST>(1.0, d[i + 1] - di) : (n > 1 ? quot_t<FIRST>(1.0, d[0] - di) : -INFINITY);
+    quad_bracket<FIRST>(b, dmin, dmax, wn2, &rlo, &rhi);
   } else {
-    double dmin = (i + 1 < n) ? quot(1.0, d[i + 1] - di) : INFINITY;
+    double dmin = (i + 1 < n) ? quot_t<FIRST>(1.0, d[i + 1] - di) : INFINITY;
     floor = fmax(-dmin, 0.0);
     // smallest delta_j: the nearest pole below d_i, or for i = n-1 the farthest pole above
-    E = (i + 1 < n) ? -dmin : (n > 1 ? quot(-1.0, d[0] - di) : -INFINITY);
+    E = (i + 1 < n) ? -dmin : (n > 1 ? quot_t<FIRST>(-1.0, d[0] - di) : -INFINITY);
     rlo = -b;
     rhi = -fmin(b, dmin) + wn;
-    if (b < dmin) rhi = fmin(rhi, -b + quot(wn2, dmin - b));
+    if (b < dmin) rhi = fmin(rhi, -b + quot_t<FIRST>(wn2, dmin - b));
     // on t = -nu the poles are -delta_j: the nearest is -dmin, the farthest -(largest delta_j)
-    const double dmx = (i > 0) ? quot(1.0, d[i - 1] - di) : (n > 1 ? quot(1.0, d[n - 1] - di) : INFINITY);
-    quad_bracket(-b, -dmx, -dmin, wn2, &rlo, &rhi);
+    const double dmx = (i > 0) ? quot_t<FIRST>(1.0, d[i - 1] - di) : (n > 1 ? quot_t<FIRST>(1.0, d[n - 1] - di) : INFINITY);
+    quad_bracket<FIRST>(-b, -dmx, -dmin, wn2, &rlo, &rhi);
   }
   alo = fmax(alo_in, rlo);
   ahi = fmin(ahi_in, rhi);
@@ -1526,7 +1531,7 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
   int steps = 0;
   double nu;
   // the finishing step's F = side g and the slope of Psi (F = side b - t + Psi)
-  const double finish = rng_ok && inv_zi2 < 0x1p100 ? (k == 0 ? kFinishCondExt : kFinishCond) : 0.0;
+  const double finish = !FIRST && rng_ok && inv_zi2 < 0x1p100 ? kFinishCond : 0.0;
   const float cf = (float)inv_zi2;
   auto fin = [&](double v, double* Fv, double* s, double* mag) -> bool {
     double S;
@@ -1539,6 +1544,13 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
     *mag = fabs(b) + fabs(S * inv_zi2);
     return isfinite(q);
   };
+  r.ill = false;
+  if (!FIRST && check && (!rng_ok || fabs(b) + mag > kIllCond * alo)) {
+    double Fv, s = 0.0, m;
+    r.ill = !rng_ok || !fin(side * ahi, &Fv, &s, &m) || fabs(b) + mag > kIllCond * alo * (1.0 + s);
+    r.steps = rng_ok;
+    if (r.ill) return r;
+  }
   uint64_t blo, bhi;
   start_bracket(&floor, alo, ahi, &blo, &bhi);
   if (fast && finish > 0.0 && bhi - blo <= kFinishWidth &&
@@ -1623,8 +1635,19 @@ __device__ PoleResult solve_pole(const double* __restrict__ d, const double* __r
   r.b = b;
   r.ok = ok;
   r.dd = used_dd;
-  r.steps = steps;
+  r.steps += steps;
   return r;
+}
+
+// The FIRST form from the shift test's pole, out of line (a few eigenvalues take it).
+template <int L, bool NI>
+__device__ __noinline__ PoleResult solve_pole_first(const double* __restrict__ d, const double* __restrict__ zl,
+                                                    const double* __restrict__ zz, int n, double rho, int k, int i,
+                                                    double alo, double ahi, int cap, bool fast, int lane, unsigned gm,
+                                                    CornerRule cr, double* __restrict__ Ds, double* __restrict__ us,
+                                                    bool screen) {
+  if (k > 0) alo = 1.0 / __dmul_rn(__dsub_rn(d[k - 1], d[k]), 0.5);
+  return solve_pole<L, NI, true>(d, zl, zz, n, rho, k, i, alo, ahi, cap, fast, lane, gm, cr, Ds, us, screen);
 }
 
 // ---------------------------------------------------------------------------------
