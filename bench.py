@@ -67,9 +67,9 @@ FP32_PER_FP64 = 64
 # the binary64 pass over the corner's terms that decides whether b needs double-double
 # (kappa_nu of Eq. (knu2)): sub, div, mul, add
 B64_OPS_PER_TERM = 4
-# the binary32 pass of the shift test (shift_test_f32): per term one binary64 subtraction and 16
-# binary32 operations (difference, reciprocal and its Newton step, quotient, w, the bound's two
-# fma, the magnitude sum, TwoSum and the low-part sum); its conversions to binary32 are integer work
+# the binary32 pass of the shift test (shift_test_f32): per term 16 binary32 operations (difference,
+# reciprocal and its Newton step, quotient, w, the bound's two fma, the magnitude sum, TwoSum and the
+# low-part sum); the poles' difference is integer work, so no binary64 operation
 SHIFT32_B64_OPS_PER_TERM = 0
 SHIFT32_OPS_PER_TERM = 16
 # an eigenvector component (Eq. (eigenvecAi)): 2 sub, 1 div, 1 mul, 1 fma (sum of squares), 1 mul
@@ -731,8 +731,8 @@ def run_ours(args):
 
     # roofline of the dominant kernel (the bisection kernel k_solve)
     evals = stats["evals_solve"]
-    # bisection steps settled by a screen or decided by a certified bound take no binary64
-    # evaluation; the screens' sums (bisection steps and probes) are binary32 work
+    # bisection steps settled by a screen, decided by a certified bound or covered by the finishing step
+    # take no binary64 evaluation; the screens' sums (bisection steps and probes) are binary32 work
     screened = stats.get("screened", 0)
     inferred = stats.get("inferred", 0)
     probes = stats.get("probes", 0)
@@ -795,13 +795,14 @@ def run_ours(args):
             "binary64_ops": ops64, "binary32_ops": ops32,
             "binary64_frac": ops64 / t_solve / NOMINAL_FP64_OPS,
             "binary32_frac": ops32 / t_solve / (FP32_PER_FP64 * NOMINAL_FP64_OPS),
-            "launch_ms": 1e3 * t_solve, "bisection_evaluations": evals,
+            "launch_ms": 1e3 * t_solve, "bisection_steps": evals,
             "binary64_evaluations": b64_evals, "screened_steps": screened, "inferred_steps": inferred,
             "screened_probes": probes, "double_float_settled": df, "double_double_corners": n_dd,
             "shift_tests_binary32": stats.get("shift_binary32", 0),
             "eigenvector_rows_written": tail_rows,
             # the plain bisection's terms (every step and the shift-test pass) per second
-            "term_rate": (n - 1) * (evals + n) / t_solve}
+            # secular terms per second in the passes that ran: evaluations, screens, shift tests
+            "term_rate": (n - 1) * (b64_evals + screened + probes + n) / t_solve}
 
     # the eigenvector phase (k_vectors and the short near-zero and deflation kernels before it):
     # the n^2 write of V against the measured copy rate, and its binary64 work against the peak

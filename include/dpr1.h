@@ -376,7 +376,7 @@ DPR1_API dpr1_status dpr1_eig_noalloc(int64_t n, const double* d, const double* 
  * out[0..17]:
  *   0 eigenvalues solved by the bisection kernel, 1 eigenvalues flagged by K_nu,
  *   2 remedies taken with R1, 3 with R2, 4 bisection steps in the bisection kernel (evaluations,
- *   and the steps of 9 and 13), 5 in the remedy kernel, 6 eigenvalues recomputed from A^{-1},
+ *   and the steps of 9 and 13: less those, the binary64 evaluations), 5 in the remedy kernel, 6 eigenvalues recomputed from A^{-1},
  *   7 deflated pairs, 8 corners b formed in double-double by the bisection kernel,
  *   9 bisection steps (of those counted in 4 and 5) settled by the binary32 screen,
  *   10 R2 remedies that formed their shift in double the working precision (of those in 3),
@@ -384,7 +384,8 @@ DPR1_API dpr1_status dpr1_eig_noalloc(int64_t n, const double* d, const double* 
  *   exceeded the screen's error bound by less than a factor 2, 12 screened evaluations (steps
  *   of 9 and probes of 14) settled by the double-float screen, 13 bisection steps (of those
  *   counted in 4 and 5) decided without an evaluation, by bounds that screened probes certified
- *   or by the finishing step that stands for the last ones, 14 screened probes that placed those bounds (not counted in 4 and 5),
+ *   or, in a solve with such bounds, by the finishing step (itself in 4 or 5) that stands for the last
+ *   ones, 14 screened probes that placed those bounds (not counted in 4 and 5),
  *   15 shift tests of the bisection kernel whose sign the binary32 pass settled (the others
  *   take the binary64 pass), 16 eigenvector rows written by the bisection kernel's lane
  *   groups after its queue ran out (the eigenvector kernel writes the others), 17 eigenvector

@@ -1157,12 +1157,13 @@ __device__ double bisect(Phi phi, double side, double floor, double alo, double 
     if (stop > 1) {
       double root;
       if (finish_root(lo, hi, side, pole, a1, finish, fin, &steps, &root)) {
-        // the steps down to adjacent doubles that this one stands for
-        const int rem = inferred ? 63 - __clzll((long long)(hi - lo)) : 0;
+        // the steps down to adjacent doubles that this one stands for, among those that certified bounds
+        // decide; without the bounds only evaluations are counted
+        const int rem = predict ? 63 - __clzll((long long)(hi - lo)) : 0;
         *ok = true;
         if (steps_out) *steps_out = steps + it + rem;
         if (screened) *screened = nscr;
-        if (inferred) *inferred = ninf + (predict ? rem : 0);
+        if (inferred) *inferred = ninf + rem;
         if (probes) *probes = nprobe;
         return root;
       }
