@@ -1396,9 +1396,10 @@ static dpr1_status run_table(const Prob& pb, void* workspace, size_t wbytes, con
   else if (L == 16) launch_solve_fix<16>(pb, w, o, grid, warps, gpw, avg_n, st);
   else launch_solve_fix<32>(pb, w, o, grid, warps, gpw, avg_n, st);
   k_zero_detect<<<sgrid, 256, 0, st>>>(pb, w, o.T_zero);
-  const int zg = pb.P < 2 * sms ? (int)pb.P : 2 * sms;   // at most one candidate per problem
-  if (avg_n > 200) k_zero_solve<256><<<zg > 0 ? zg : 1, 256, 0, st>>>(pb, w, o.cap, o.fast);
-  else k_zero_solve<32><<<zg > 0 ? zg : 1, 32, 0, st>>>(pb, w, o.cap, o.fast);
+  int64_t zg = pb.P < 2 * sms ? pb.P : 2 * sms;          // at most one candidate per problem
+  if (w.terms && zg > w.term_slots) zg = w.term_slots;   // every group with a buffer
+  if (avg_n > 200) k_zero_solve<256><<<zg > 0 ? (int)zg : 1, 256, 0, st>>>(pb, w, o.cap, o.fast);
+  else k_zero_solve<32><<<zg > 0 ? (int)zg : 1, 32, 0, st>>>(pb, w, o.cap, o.fast);
   k_defl_positions<<<sgrid, 256, 0, st>>>(pb, w);
   int64_t vg = (pb.total + 7) / 8;
   if (vg > sms * 16) vg = sms * 16;
