@@ -409,6 +409,15 @@ DPR1_API dpr1_status dpr1_probe_dfma(int blocks, int threads, int iters, double*
  */
 DPR1_API dpr1_status dpr1_probe_reciprocal(int64_t count, const double* x, double* out, dpr1_stream_t stream);
 
+/*
+ * Test hook: out[t] = one of the library's scalar operations for t < count, `which` 0: the reciprocal
+ * 1/a of the term loops, 1: the reciprocal of the secular function's evaluations, 2: the quotient a/b and
+ * 3: the rough quotient a/b of the brackets and corrections, 4: the square root of a, 5: |a| truncated to
+ * binary32.  b is read for 2 and 3 only.
+ */
+DPR1_API dpr1_status dpr1_probe_scalar(int which, int64_t count, const double* a, const double* b, double* out,
+                                       dpr1_stream_t stream);
+
 #ifdef __cplusplus
 }
 #endif

@@ -63,6 +63,8 @@ def lib():
         L.dpr1_stream_status.restype = ctypes.c_int
         L.dpr1_probe_reciprocal.argtypes = [_i64, _vp, _vp, _vp]
         L.dpr1_probe_reciprocal.restype = ctypes.c_int
+        L.dpr1_probe_scalar.argtypes = [ctypes.c_int, _i64, _vp, _vp, _vp, _vp]
+        L.dpr1_probe_scalar.restype = ctypes.c_int
         L.dpr1_workspace_stats.argtypes = [_vp, ctypes.POINTER(ctypes.c_int64), _vp]
         L.dpr1_workspace_stats.restype = ctypes.c_int
         L.dpr1_probe_dfma.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, _vp, _vp]
@@ -269,6 +271,16 @@ def probe_reciprocal(x):
     x = _dev_f64(x, torch.device("cuda", torch.cuda.current_device()))
     out = torch.empty_like(x)
     _check(lib().dpr1_probe_reciprocal(x.numel(), _ptr(x), _ptr(out), _stream()), "dpr1_probe_reciprocal")
+    torch.cuda.synchronize()
+    return out
+
+
+def probe_scalar(which, a, b=None):
+    dev = torch.device("cuda", torch.cuda.current_device())
+    a = _dev_f64(a, dev)
+    b = _dev_f64(b, dev) if b is not None else None
+    out = torch.empty_like(a)
+    _check(lib().dpr1_probe_scalar(which, a.numel(), _ptr(a), _ptr(b), _ptr(out), _stream()), "dpr1_probe_scalar")
     torch.cuda.synchronize()
     return out
 

@@ -1230,6 +1230,15 @@ __global__ void k_probe_rcp(int64_t count, const double* __restrict__ x, double*
     out[t] = rcp(x[t]);
 }
 
+__global__ void k_probe_scalar(int which, int64_t count, const double* __restrict__ a, const double* __restrict__ b,
+                               double* __restrict__ out) {
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < count; t += (int64_t)gridDim.x * blockDim.x) {
+    const double x = a[t];
+    out[t] = which == 0 ? rcp(x) : which == 1 ? rcp_c(x) : which == 2 ? quot(x, b[t]) : which == 3 ? quot_approx(x, b[t])
+             : which == 4 ? root(x) : (double)mag_f32(x);
+  }
+}
+
 // ---------------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------------
@@ -1565,6 +1574,16 @@ dpr1_status dpr1_workspace_stats(void* workspace, int64_t* out, dpr1_stream_t st
 dpr1_status dpr1_probe_dfma(int blocks, int threads, int iters, double* sink, dpr1_stream_t stream) {
   if (blocks <= 0 || threads <= 0 || threads > 1024 || iters <= 0 || !sink) return DPR1_ERR_ARG;
   k_probe_dfma<<<blocks, threads, 0, (cudaStream_t)stream>>>(iters, sink);
+  return cudaGetLastError() == cudaSuccess ? DPR1_OK : DPR1_ERR_CUDA;
+}
+
+dpr1_status dpr1_probe_scalar(int which, int64_t count, const double* a, const double* b, double* out,
+                              dpr1_stream_t stream) {
+  if (which < 0 || which > 5 || count < 0 || (count > 0 && (!a || !out || ((which == 2 || which == 3) && !b))))
+    return DPR1_ERR_ARG;
+  if (count == 0) return DPR1_OK;
+  const int64_t g = (count + 255) / 256;
+  k_probe_scalar<<<(int)(g < 4096 ? g : 4096), 256, 0, (cudaStream_t)stream>>>(which, count, a, b, out);
   return cudaGetLastError() == cudaSuccess ? DPR1_OK : DPR1_ERR_CUDA;
 }
 
