@@ -194,7 +194,8 @@ __global__ void __launch_bounds__(32 * WPB, 1) k_bwd_rows(int n, double rho_in, 
     const double xp = __dmul_rn(z[p], rp);
     const double gvp = grow ? grow[p] : 0.0;
     double cv, nrm;                            // v_j = x_j cv, cv = 1 / ||x||
-    if (mx > 1e-70 && mx < 1e100 && isfinite(S2) && isfinite(P) && isfinite(A) && isfinite(Bs)) {
+    // in units of x, no further from underflow than 2^-120 of the cotangents; overflow shows in the sums
+    if (mx > 0x1p-60 && mx < 1e100 && isfinite(S2) && isfinite(P) && isfinite(A) && isfinite(Bs)) {
       nrm = sqrt(__fma_rn(xp, xp, S2));
       cv = 1.0 / nrm;
       const double c2 = cv * cv;
