@@ -103,6 +103,7 @@ enum : unsigned {
 constexpr size_t TERM_BYTES = 32;
 
 size_t ws_layout(int64_t n, Ws* w, char* base);
+size_t ws_layout2(int64_t total, int64_t nprob, bool batched, Ws* w, char* base);
 size_t term_bytes(int64_t total, int64_t nprob);
 Options resolve(const dpr1_options* o);
 int sm_count();

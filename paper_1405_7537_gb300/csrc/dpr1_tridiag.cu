@@ -34,9 +34,6 @@
 
 namespace dpr1 {
 
-// the workspace layout of a batched call (dpr1_eig.cu)
-size_t ws_layout2(int64_t total, int64_t nprob, bool batched, Ws* w, char* base);
-
 static size_t a256t(size_t x) { return (x + 255) & ~(size_t)255; }
 
 static int tree_depth(int64_t n) {
