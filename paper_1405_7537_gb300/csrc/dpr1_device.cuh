@@ -7,9 +7,10 @@
 //   TwoSum, Dekker's FastTwoSum and the exact product through fma.
 // * a binary64 reciprocal within one unit in the last place of 1/x for |x| in
 //   [2^-1020, 2^1020] (outside that range the IEEE quotient is used): a Newton step on a
-//   seed from binary32 and integer arithmetic (the loops over the terms), or one
-//   third-order step r = r0 (1 + e + e^2), e = 1 - x r0, on the sm_103a approximate
-//   reciprocal instruction (rcp.approx.ftz.f64, about 20 correct bits).
+//   seed from binary32 and integer arithmetic (the elements, the eigenvectors, the
+//   adjoint), or one third-order step r = r0 (1 + e + e^2), e = 1 - x r0, on the sm_103a
+//   approximate reciprocal instruction (rcp.approx.ftz.f64, about 20 correct bits: the
+//   evaluations, the scalar work and the elements of ill-conditioned eigenvalues).
 // * lane-group reductions with xor shuffles: every lane of a group ends with the
 //   bit-identical total (IEEE addition is commutative), so every lane takes the
 //   same bisection decisions without a broadcast.
@@ -84,7 +85,8 @@ __device__ __forceinline__ float rcp_approx_f32(float x) {
 }
 
 // 1/x within one ulp for |x| in [2^-1020, 2^1021) (see the file comment); no range handling.  The
-// shortest chain, for the scalar work.
+// shortest chain, for the scalar work; and the arithmetic of ill-conditioned first solves (solve_pole),
+// which is part of their result.
 __device__ __forceinline__ double rcp_chain(double x) {
   double r0 = rcp_approx(x);
   double e = __fma_rn(-x, r0, 1.0);

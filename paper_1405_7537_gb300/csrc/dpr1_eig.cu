@@ -152,9 +152,9 @@ size_t ws_layout2(int64_t total, int64_t nprob, bool batched, Ws* w, char* base)
 // the GPU idle (whole call, us, packed and a warp each: n = 200 280 and 264, n = 384 395 and 386).
 // With 32 lanes n = 96 takes 180 us against 226: the exterior eigenvalue's
 // solve, 8 lanes wide, is the longest.  In a batch, eight lanes up to a mean order of 384 (problems of
-// orders 96-384: 33.3 ms against 39.8 with 16 lanes and 48.3 with 32 for 425k eigenpairs; orders 16-96: 18.2
-// against 24.9 and 32.5, with the solver of that time, half as fast) and a warp above (orders 384-2048:
-// 108.4 ms against 115.8 with 16 lanes and 140.3 with 8).
+// orders 96-384: 16.8 ms against 19.5 with 16 lanes and 21.2 with 32 for 415k eigenpairs; orders 16-96: 8.7
+// against 11.4 and 13.5 for 358k) and a warp above (orders 384-2048: 54.2 ms against 59.6 with 16 lanes and
+// 78.9 with 8 for 504k).
 static int default_lanes(double avg_n, int64_t nprob = 1) {
   if (nprob > 1) return avg_n <= 384 ? 8 : 32;
   return avg_n <= 96 ? 8 : (avg_n <= 384 ? 16 : 32);

@@ -966,8 +966,8 @@ __device__ __forceinline__ void start_bracket(double* floor, double alo, double 
 // (its tolerance covers the screen's error, the bound and the roundings); hence every t below a
 // point settled "below" (above a point settled "above") gets phi's decision "below" ("above")
 // without an evaluation.  With `predict`, screened probes set such bounds cl and ch next to the
-// root: from the upper end, the accelerated solve's pole model (model_root: pole `pole`, F =
-// a0 - t + Psi) fitted to each probe's screened value and slope gives the next probe, first with
+// root: from the upper end, the accelerated solve's pole model (placed in binary32 by model_point: pole
+// `pole`, F = a0 - t + Psi) fitted to each probe's screened value and slope gives the next probe, first with
 // the binary32 screen, then, once its steps shrink below twice its tolerance over the slope (or
 // it cannot settle a probe), with the double-float screen; one double-float step later two probes
 // at that estimate minus and plus twice the tolerance over the slope certify both sides.  The
